@@ -881,7 +881,7 @@ int g6x_open_ex(int cid, int nj_max, int ni_max)
     js.j664 = (double4_32a *)dev_alloc(n * sizeof(double4_32a));
     js.idx = (int *)dev_alloc(n * sizeof(int));
     c.pred.pt = (float *)dev_alloc(n * g6::JW * sizeof(float));
-    c.pred.trange = (int2 *)dev_alloc((n / JT) * sizeof(int2));
+    c.pred.trange = (int2 *)dev_alloc((n / JT) * g6::NRANGE * sizeof(int2));
     c.pred.p64 = (double4_32a *)dev_alloc(n * sizeof(double4_32a));
     c.pred.v64 = (double4_32a *)dev_alloc(n * sizeof(double4_32a));
     {

@@ -645,7 +645,7 @@ g6x_batch *g6x_batch_create(int ncl, const int nj[], int precision, int variant,
     js.j664 = dalloc<double4_32a>(n);
     js.idx = dalloc<int>(n);
     b->pred.pt = dalloc<float>(n * g6::JW);
-    b->pred.trange = dalloc<int2>(tiles);
+    b->pred.trange = dalloc<int2>(tiles * g6::NRANGE);
     b->d_tile_cluster = dalloc<int>(tiles);
     b->d_cl_jtile = dalloc<int>(ncl);
     b->d_cl_nj = dalloc<int>(ncl);

@@ -297,9 +297,59 @@ __device__ __forceinline__ void far_slot_ds(float *o)
     o[W_ID * JT] = __int_as_float(-1);
 }
 
+// The j-particle with the smallest key in a share of a tile (share = tile x
+// SHT + group, the groups' shares contiguous), by SL neighbouring lanes of a
+// warp that call this together: they take the share's j-particles side by
+// side, so that their loads coalesce (scan), and agree on the first j with
+// the smallest key (agree).  key_of(tile, jj, id) is the loop's own key of
+// j-particle jj of a tile (+inf for the i-particle's own j and for empty
+// slots) and its particle index.  Two steps, so that the loads of several
+// searches are in flight before the first one agrees.
+template <int SHT>
+struct ShareSearch {
+    static constexpr int SHJ = JT / SHT;              // j-particles of a share
+    static constexpr int SL = SHJ < 32 ? SHJ : 32;    // lanes that search together
+    float best;
+    int bj, bid;                                      // the lane's best: j-slot, index
+    template <class Key>
+    __device__ __forceinline__ void scan(int share, Key key_of)
+    {
+        best = __int_as_float(0x7f800000);
+        bj = INT_MAX;
+        bid = -1;
+        if (share < 0)
+            return;
+        const int tile = share / SHT, j0 = (share % SHT) * SHJ + (threadIdx.x & 31) % SL;
+#pragma unroll
+        for (int r = 0; r < SHJ / SL; ++r) {
+            const int jj = j0 + r * SL;
+            int id = -1;
+            const float key = key_of(tile, jj, id);
+            if (key < best) {
+                best = key;
+                bj = tile * JT + jj;
+                bid = id;
+            }
+        }
+    }
+    // The winner's j-slot (INDEX false) or particle index, -1 if the share
+    // has no finite key.
+    template <bool INDEX>
+    __device__ __forceinline__ int agree() const
+    {
+        const int sub = (threadIdx.x & 31) / SL * SL;
+        const unsigned lanes = SL == 32 ? 0xffffffffu : ((1u << (SL & 31)) - 1u) << sub;
+        const unsigned kmin = __reduce_min_sync(lanes, __float_as_uint(best));
+        const int won = __reduce_min_sync(lanes, __float_as_uint(best) == kmin ? bj : INT_MAX);
+        if constexpr (!INDEX)
+            return won == INT_MAX ? -1 : won;
+        return __reduce_max_sync(lanes, won != INT_MAX && bj == won ? bid : -1);
+    }
+};
+
 struct ForceArgs {
     const float *pt;                  // DS predicted j, tiled layout
-    const int2 *trange;               // DS per-tile index range
+    const int2 *trange;               // DS index ranges, NRANGE per tile
     const double4_32a *p64, *v64;         // FP64 predicted j
     const g6x_irec *irec;
     void *part;                       // PartialDS (DS kernels) or Partial64 (FP64)

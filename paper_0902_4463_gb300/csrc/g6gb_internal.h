@@ -81,13 +81,16 @@ struct JStore {
 constexpr int JW = 11;
 enum JWord { W_XH = 0, W_YH, W_ZH, W_M, W_XL, W_YL, W_ZL, W_VX, W_VY, W_VZ, W_ID };
 
+// Index ranges kept per tile: one per 32 j-slots.
+constexpr int NRANGE = JT / 32;
+
 // Predicted j-particles (force-kernel input).
 struct Pred {
     float *pt;         // DS: tiled layout above, cap / JT tiles
-    int2 *trange;      // DS: per tile, smallest and largest particle index
-                       //     (empty tile: INT_MAX, -1); lets the force kernel
-                       //     skip the per-pair self test on tiles that hold
-                       //     none of its i-particles
+    int2 *trange;      // DS: per 32 j-slots (NRANGE per tile), smallest and largest
+                       //     particle index (none: INT_MAX, -1); lets a warp of the
+                       //     force kernel skip the per-pair self test where its
+                       //     share of a tile holds none of its i-particles
     double4_32a *p64;      // FP64: (x, y, z, m)
     double4_32a *v64;      // FP64: (vx, vy, vz, index)
 };

@@ -96,30 +96,15 @@ __global__ void k_irec_from_store(JStore js, g6x_irec *out, int m)
 // ----------------------------------------------------------------- K1 ---
 
 
-// Records one tile's range of particle indices (empty slots excluded);
-// called by all JT threads of the CTA with their own slot's index.  The
-// per-warp ranges go to the half `par` of the double-buffered s_lo / s_hi,
-// so consecutive tiles need only the one barrier here: the next tile writes
-// the other half, and the tile after that passes this tile's barrier after
-// thread 0 has read its half.
-__device__ __forceinline__ void tile_index_range(int (*s_lo)[JT / 32], int (*s_hi)[JT / 32],
-                                                 int par, int id, bool valid, int2 *out)
+// Records the range of particle indices of each 32 j-slots (empty slots
+// excluded): every warp of the CTA its own, so the predictor needs no
+// barrier (with one range per tile it met at one per tile).
+__device__ __forceinline__ void index_ranges(int id, bool valid, int2 *out)
 {
-    int lo_id = valid ? id : INT_MAX, hi_id = valid ? id : -1;
-    lo_id = __reduce_min_sync(0xffffffffu, lo_id);
-    hi_id = __reduce_max_sync(0xffffffffu, hi_id);
-    if ((threadIdx.x & 31) == 0) {
-        s_lo[par][threadIdx.x >> 5] = lo_id;
-        s_hi[par][threadIdx.x >> 5] = hi_id;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < JT / 32; ++w) {
-            lo_id = min(lo_id, s_lo[par][w]);
-            hi_id = max(hi_id, s_hi[par][w]);
-        }
-        *out = make_int2(lo_id, hi_id);
-    }
+    const int lo = __reduce_min_sync(0xffffffffu, valid ? id : INT_MAX);
+    const int hi = __reduce_max_sync(0xffffffffu, valid ? id : -1);
+    if ((threadIdx.x & 31) == 0)
+        out[threadIdx.x >> 5] = make_int2(lo, hi);
 }
 
 // Eq. 1 and Eq. 2 for one j-slot k < nj in the paper's DS + SP form
@@ -184,17 +169,15 @@ __device__ __forceinline__ void predict_slot_64(const JStore &js, Pred &p, int k
 // (rec sorted by tile, tile t's records at [toff[t], toff[t+1])) -- the K0
 // update fused into the same launch -- then predicts the tile.  Tiles at or
 // beyond the predicted range only take their updates.  The DS kinds also
-// record each tile's range of particle indices.
+// record the range of particle indices of each 32 slots.
 template <int KIND, bool UPD>
 __global__ void __launch_bounds__(JT) k_predict(JStore js, Pred p, int nj, int nj_pad,
                                                 double t, const g6x_jrec *__restrict__ rec,
                                                 const int *__restrict__ toff, int ntiles_all)
 {
     grid_dep_launch();              // the force kernel may be scheduled behind this one
-    __shared__ int s_lo[2][JT / 32], s_hi[2][JT / 32];
     const int ntiles_pred = nj_pad / JT;
     const int ntiles = UPD ? ntiles_all : ntiles_pred;
-    int par = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         if constexpr (UPD) {
             for (int r = toff[tile] + threadIdx.x; r < toff[tile + 1]; r += JT)
@@ -209,8 +192,7 @@ __global__ void __launch_bounds__(JT) k_predict(JStore js, Pred p, int nj, int n
         } else {
             float *o = p.pt + (size_t)tile * (JW * JT) + threadIdx.x;
             const int id = k < nj ? js_idx(js, k) : -1;
-            tile_index_range(s_lo, s_hi, par, id, k < nj && id >= 0, &p.trange[tile]);
-            par ^= 1;
+            index_ranges(id, k < nj && id >= 0, &p.trange[(size_t)tile * NRANGE]);
             if (k >= nj)
                 far_slot_ds(o);
             else if constexpr (KIND == PRED_DS)
@@ -228,8 +210,6 @@ __global__ void __launch_bounds__(JT) k_predict_batch(JStore js, Pred p, BatchPr
                                                       const int *__restrict__ toff, int tile0,
                                                       int ntiles)
 {
-    __shared__ int s_lo[2][JT / 32], s_hi[2][JT / 32];
-    int par = 0;
     for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x) {
         const int tile = tile0 + tt;
         if (rec && toff) {
@@ -249,8 +229,7 @@ __global__ void __launch_bounds__(JT) k_predict_batch(JStore js, Pred p, BatchPr
         } else {
             float *o = p.pt + (size_t)tile * (JW * JT) + threadIdx.x;
             const int id = valid ? js_idx(js, slot) : -1;
-            tile_index_range(s_lo, s_hi, par, id, valid && id >= 0, &p.trange[tile]);
-            par ^= 1;
+            index_ranges(id, valid && id >= 0, &p.trange[(size_t)tile * NRANGE]);
             if (!valid)
                 far_slot_ds(o);
             else if constexpr (KIND == PRED_DS)
@@ -304,12 +283,17 @@ __device__ __forceinline__ float2 ds_sep2(float2 h, float2 l, float2 nh, float2 
 // issue two lanes of FP32 work per instruction.  Subtractions are additions
 // of the pre-negated i values (exact).
 //
-// The per-pair self test is needed only on j-tiles whose index range holds
-// one of the warp's i-particles; other tiles take the same loop without it.
+// The j-groups take contiguous shares of a tile, so that the loads of two
+// j-pairs merge into 16-byte ones (strided shares: 3-7 % slower) and a
+// group's j-slots ascend; batches, whose entries are short, keep strided
+// shares.  The per-pair self test is needed only where the
+// index range of a warp's j-particles holds one of its i-particles; others
+// take the same loop without it.
 // The nearest neighbour is tracked lazily: a running minimum of the key per
-// tile and the tile that lowered it; when a segment ends, that one tile is
-// scanned again with the same arithmetic to find the first j that attains
-// the minimum (ties to the lower j-slot).  Lists (Sect. 4) use the same
+// tile and the share (tile x group) that lowered it; when a segment ends,
+// the winning share of each i-particle is scanned again with the same
+// arithmetic to find the first j that attains the minimum (ties to the lower
+// j-slot).  Lists (Sect. 4) use the same
 // minimum: the loop keeps it per chunk of j-pairs, and only a chunk whose
 // minimum is below h2 + eps2 is scanned again, from the staged tile, for
 // its members, so the pair loop is the same with and without lists.  With
@@ -329,14 +313,18 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
     constexpr int NT = TI * TJ;
     constexpr int ITILE = TI * NI;
     constexpr int PPT = JT / 2 / TJ;                  // j-pairs per thread per tile
+    // Shares of a tile: group g's j-pairs are g * PPT + kk (contiguous), or
+    // g + kk * TJ in batches.  SHT: shares per tile that are searched for the
+    // nearest neighbour (the contiguous ones, or the whole tile where shares
+    // interleave, so that ties go to the lower j-slot).
+    constexpr bool STRIDED = BATCH;
+    constexpr int SHT = STRIDED ? 1 : TJ;
+    constexpr int SHJ = JT / SHT;
     constexpr int FLUSH = (256 + PPT - 1) / PPT;      // tiles between flushes (>= 512 j)
-    // The split-j shapes (small m) also note which chunk of CHP j-pairs
-    // lowered a tile's minimum, so the rescan at the end of a segment reads
-    // one chunk of the winning tile, not the thread's whole share of it.
     // Lists test each chunk's minimum against the radius: whole j-tiles per
-    // thread take chunks of 16 j-pairs (4 cost the loop 8 %).
-    constexpr bool NNC = TJ > 1;
-    constexpr int CHW = NNC ? 4 : 16;
+    // thread take chunks of 16 j-pairs (4 cost the loop 8 %), the split-j
+    // shapes chunks of 4.
+    constexpr int CHW = TJ > 1 ? 4 : 16;
     constexpr int CHP = PPT < CHW ? PPT : CHW;
     static_assert(PPT % CHP == 0, "whole chunks per tile");
     constexpr unsigned TILE_BYTES = JW * JT * sizeof(float);
@@ -366,9 +354,10 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
     __shared__ int s_nbn[LRUN ? NI * NT : 1];
     __shared__ int s_nbh[LRUN ? NI * NT : 1];
     __shared__ float s_ibuf[TJ > 1 ? 11 * ITILE : 1];
+    __shared__ int s_win[TJ > 1 ? ITILE : 1];        // winning share per i-particle
 
-    const int tid = threadIdx.x;
-    const int ti = tid % TI, tj = tid / TI;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int ti = tid % TI, tj = TJ > 1 ? tid / TI : 0;
     const long long G = gridDim.x, c = blockIdx.x;
     // Work geometry: global i-tile g of a work position, its work range, its
     // j-tile for a position, and where its i-records and results live.
@@ -511,8 +500,7 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
     int iid[NI];
     float2 ta[NI][7];
     float tmin[NI], nnr[NI];
-    int nnt[NI], nbn[NI];
-    int tchk[NI], nnc[NI];              // NNC: chunk of the tile / of tile nnt
+    int nnt[NI], nbn[NI];               // nnt: the share (tile x group) with the smallest key
     int cur_t = -1;
     int since_flush = 0;
 
@@ -618,75 +606,59 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
             nnr[k] = INF;
             nnt[k] = -1;
             nbn[k] = 0;
-            tchk[k] = 0;
-            nnc[k] = 0;
         }
         since_flush = 0;
         if constexpr (TJ > 1)
             __syncthreads();          // s_ibuf is reused by the next segment
     };
 
-    // First j of the thread's share of tile nnt[k] whose key equals nnr[k],
-    // recomputed with the loop's arithmetic (packed lanes round like the
-    // scalar operations used here).  The loads of 8 j-particles are issued
-    // together so the rescan costs a few memory latencies, not one per j.
-    auto nn_rescan = [&](int k) -> int {
-        if (!(nnr[k] < INF) || nnt[k] < 0)
-            return -1;
-        const float *T = a.pt + (size_t)nnt[k] * JW * JT;
-        constexpr int CH = NNC ? CHP : 4;           // j-pairs loaded together
-        const int kb = NNC ? nnc[k] * CH : 0, ke = NNC ? kb + CH : PPT;
-        for (int kk0 = kb; kk0 < ke; kk0 += CH) {
-            float key[2 * CH];
-#pragma unroll
-            for (int u = 0; u < CH; ++u) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int kk = kk0 + u;
-                    const int jj = 2 * (tj + kk * TJ) + h;
-                    float r2u = INF;
-                    int id = -1;
-                    // FP: the tile was never stored; predict this j again
-                    // with the same arithmetic (empty slots cannot win)
-                    const int slot = nnt[k] * JT + jj;
-                    if (kk < PPT && (!FP || slot < a.nj)) {
-                        float ph[3], pl[3];
-                        if constexpr (FP) {
-                            const float hh = (float)(a.t_pred - js_t0(a.js, slot));
-                            predict_ds_pos(hh, js_xds(a.js, slot), js_xds2(a.js, slot),
-                                           js_v0m(a.js, slot), js_a2f(a.js, slot),
-                                           js_j6f(a.js, slot), ph, pl);
-                            id = js_idx(a.js, slot);
-                        } else {
-                            ph[0] = __ldg(T + W_XH * JT + jj);
-                            ph[1] = __ldg(T + W_YH * JT + jj);
-                            ph[2] = __ldg(T + W_ZH * JT + jj);
-                            pl[0] = __ldg(T + W_XL * JT + jj);
-                            pl[1] = __ldg(T + W_YL * JT + jj);
-                            pl[2] = __ldg(T + W_ZL * JT + jj);
-                            id = __float_as_int(__ldg(T + W_ID * JT + jj));
-                        }
-                        // the loop's own separation arithmetic, lane by lane
-                        float dd[3];
-#pragma unroll
-                        for (int d = 0; d < 3; ++d) {
-                            if constexpr (DSS)
-                                dd[d] = ds_sep1(ph[d], pl[d], nxh[k][d].x, nxl[k][d].x);
-                            else
-                                dd[d] = __fadd_rn(__fadd_rn(ph[d], nxh[k][d].x),
-                                                  __fadd_rn(pl[d], nxl[k][d].x));
-                        }
-                        r2u = soft_r2(dd[0], dd[1], dd[2], eps2.x);
-                    }
-                    key[2 * u + h] = (id == iid[k]) ? INF : r2u;
-                }
+    // Nearest neighbour of one i-particle (negated DS position xh, xl, index
+    // id_i) from the share that holds its smallest key, by SL lanes together:
+    // the keys again with the loop's arithmetic, whose packed lanes round
+    // like the scalar operations used here.  (Before, every thread searched
+    // the chunk of 8 j-particles noted in the loop for each of its own
+    // i-particles, before the j-groups were combined: scattered loads that
+    // took 25 of the 350 us of m = 251, N = 10^6, and the notes cost the
+    // loop 4 %.)
+    using Search = ShareSearch<SHT>;
+    constexpr int SL = Search::SL;
+    auto nn_scan = [&](int share, const float *xh, const float *xl, int id_i) -> Search {
+        auto key_of = [&](int tile, int jj, int &id) -> float {
+            // FP: the tile was never stored; predict this j again with the
+            // same arithmetic
+            float ph[3], pl[3];
+            if constexpr (FP) {
+                const int slot = tile * JT + jj;
+                if (slot >= a.nj)
+                    return INF;
+                predict_ds_pos((float)(a.t_pred - js_t0(a.js, slot)), js_xds(a.js, slot),
+                               js_xds2(a.js, slot), js_v0m(a.js, slot), js_a2f(a.js, slot),
+                               js_j6f(a.js, slot), ph, pl);
+                id = js_idx(a.js, slot);
+            } else {
+                const float *T = a.pt + (size_t)tile * JW * JT;
+                ph[0] = __ldg(T + W_XH * JT + jj);
+                ph[1] = __ldg(T + W_YH * JT + jj);
+                ph[2] = __ldg(T + W_ZH * JT + jj);
+                pl[0] = __ldg(T + W_XL * JT + jj);
+                pl[1] = __ldg(T + W_YL * JT + jj);
+                pl[2] = __ldg(T + W_ZL * JT + jj);
+                id = __float_as_int(__ldg(T + W_ID * JT + jj));
             }
+            float dd[3];
 #pragma unroll
-            for (int u = 0; u < 2 * CH; ++u)
-                if (key[u] == nnr[k])
-                    return nnt[k] * JT + 2 * (tj + (kk0 + u / 2) * TJ) + (u & 1);
-        }
-        return -1;
+            for (int d = 0; d < 3; ++d) {
+                if constexpr (DSS)
+                    dd[d] = ds_sep1(ph[d], pl[d], xh[d], xl[d]);
+                else
+                    dd[d] = __fadd_rn(__fadd_rn(ph[d], xh[d]), __fadd_rn(pl[d], xl[d]));
+            }
+            const float key = soft_r2(dd[0], dd[1], dd[2], eps2.x);
+            return id == id_i ? INF : key;
+        };
+        Search w;
+        w.scan(share, key_of);
+        return w;
     };
 
     // Reduction of i-tile t by the last CTA that finished it (Sect. 2.3:
@@ -834,7 +806,22 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
                 }
                 P->pot = cslot(k, 6);
                 P->nnr2 = unsoftened(nnr[k], eps2.x);
-                P->nnj = nn_rescan(k);
+                // each of the warp's i-particles in turn, by the whole warp
+                int nnj = -1;
+                for (int l = 0; l < 32; ++l) {
+                    float xh[3], xl[3];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        xh[d] = __shfl_sync(0xffffffffu, nxh[k][d].x, l);
+                        xl[d] = __shfl_sync(0xffffffffu, nxl[k][d].x, l);
+                    }
+                    const int j = nn_scan(__shfl_sync(0xffffffffu, nnt[k], l), xh, xl,
+                                          __shfl_sync(0xffffffffu, iid[k], l))
+                                      .template agree<false>();
+                    if (lane == l)
+                        nnj = j;
+                }
+                P->nnj = nnj;
                 if constexpr (LIST) {
                     a.nbc[(size_t)seg * ITILE + il] = nbn[k];
                     if (nbn[k] > 0)
@@ -842,14 +829,16 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
                 }
             }
         } else {
-            // The TJ j-groups of an i-particle combine in place: every
-            // thread's compensated sums are in comp[], its nearest neighbour
-            // goes to s_nnr / s_nnj, and one thread per i-particle adds the
-            // groups in compensated FP32 (neighbour ties to the lower j-slot).
+            // The j-groups of an i-particle combine in place: every thread's
+            // compensated sums are in comp[], its smallest key and the share
+            // that holds it go to s_nnr / s_nnj, and one thread per
+            // i-particle adds the groups in compensated FP32 (neighbour ties
+            // to the lower share or tile, which holds the lower j-slots).  Then
+            // SL lanes per i-particle search the winning share.
 #pragma unroll
             for (int k = 0; k < NI; ++k) {
                 s_nnr[k * NT + tid] = nnr[k];
-                s_nnj[k * NT + tid] = nn_rescan(k);
+                s_nnj[k * NT + tid] = nnt[k];
                 if constexpr (LRUN)
                     s_nbn[k * NT + tid] = nbn[k];
             }
@@ -886,9 +875,9 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
                 }
                 P->pot = make_float2(sh[6], sl[6]);
                 P->nnr2 = unsoftened(br, eps2.x);
-                P->nnj = bj;
+                s_win[il] = bj;
                 if constexpr (LRUN) {
-                    // merge the TJ ascending runs into the list partial;
+                    // merge the ascending runs into the list partial;
                     // a run keeps its first nbseg entries, and a total above
                     // nbseg makes the host compute the lists again with more
                     // room, unless nbseg is already the list length (then
@@ -926,13 +915,39 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
                 }
             }
             __syncthreads();
+            constexpr int SPR = NT / SL;              // i-particles searched per round
+            constexpr int SW = ITILE > 2 * SPR ? 4 : ITILE > SPR ? 2 : 1;   // rounds in flight
+            static_assert(ITILE % (32 / SL) == 0, "whole warps search together");
+            for (int i0 = tid / SL; i0 < ITILE; i0 += SW * SPR) {
+                Search w[SW];
+#pragma unroll
+                for (int r = 0; r < SW; ++r) {
+                    const int il = i0 + r * SPR, is = il < ITILE ? il : i0;
+                    float xh[3], xl[3];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        xh[d] = -s_ibuf[d * ITILE + is];
+                        xl[d] = -s_ibuf[(3 + d) * ITILE + is];
+                    }
+                    w[r] = nn_scan(il < ITILE ? s_win[is] : -1, xh, xl,
+                                   __float_as_int(s_ibuf[10 * ITILE + is]));
+                }
+#pragma unroll
+                for (int r = 0; r < SW; ++r) {
+                    const int il = i0 + r * SPR, j = w[r].template agree<false>();
+                    if (lane % SL == 0 && il < ITILE)
+                        PP[(size_t)seg * ITILE + il].nnj = j;
+                }
+            }
+            __syncthreads();
         }
         if (a.fused)
             tile_done(t);
     };
 
     // All pairs of the thread's share of one staged tile.  SELF: apply the
-    // per-pair self test (tiles that may hold one of the i-particles).
+    // per-pair self test (where the warp's j-particles may hold one of its
+    // i-particles).
     auto tile_pass = [&](const float *S, int t, int jt, auto self_tag) {
         constexpr bool SELF = decltype(self_tag)::value;
         const float2 *XH = reinterpret_cast<const float2 *>(S + W_XH * JT);
@@ -949,7 +964,7 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
         // j-pair kk of the thread's share against its NI i-particles; mins[k]
         // receives the smaller key
         auto jpair = [&](int kk, float (&mins)[NI]) {
-            const int jp = tj + kk * TJ;
+            const int jp = STRIDED ? tj + kk * TJ : tj * PPT + kk;
             const float2 xh = XH[jp], yh = YH[jp], zh = ZH[jp], mj = MM[jp];
             const float2 xl = XL[jp], yl = YL[jp], zl = ZL[jp];
             const float2 vx = VX[jp], vy = VY[jp], vz = VZ[jp];
@@ -1003,7 +1018,7 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
         auto list_chunk = [&](int ch, int k) {
             int *dst = list_run(c + t, k * TI + ti, tj);
             for (int u = 0; u < CHP; ++u) {
-                const int jp = tj + (ch * CHP + u) * TJ;
+                const int jp = tj * PPT + ch * CHP + u;
                 const float2 xh = XH[jp], yh = YH[jp], zh = ZH[jp];
                 const float2 xl = XL[jp], yl = YL[jp], zl = ZL[jp];
                 const int2 id = ID[jp];
@@ -1031,7 +1046,7 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
                 }
             }
         };
-        if constexpr (NNC || LIST) {
+        if constexpr (LIST) {
             for (int ch = 0; ch < PPT / CHP; ++ch) {
                 float cm[NI];
 #pragma unroll
@@ -1042,13 +1057,9 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
                     jpair(ch * CHP + u, cm);
 #pragma unroll
                 for (int k = 0; k < NI; ++k) {
-                    if constexpr (LIST)
-                        if (cm[k] < h2[k])
-                            list_chunk(ch, k);
-                    if (cm[k] < tmin[k]) {      // the first chunk that reaches the minimum
-                        tmin[k] = cm[k];
-                        tchk[k] = ch;
-                    }
+                    if (cm[k] < h2[k])
+                        list_chunk(ch, k);
+                    tmin[k] = fminf(tmin[k], cm[k]);
                 }
             }
         } else {
@@ -1059,12 +1070,46 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
     };
 
     int cur_g = g_of(wb);
+    int jt_next = jt_of(wb, cur_g);              // AHEAD: the next tile and its range
+    // The index range of the j-particles that the warp walks in a tile: its
+    // groups' contiguous shares (one or two ranges of 32), or with whole
+    // tiles and strided shares all NRANGE of them, a lane each.  Ranges of 32
+    // keep the self test off all but the shares that need it: with one range
+    // per tile, a quarter of the tiles took it at N = 32768.  The split-j
+    // shapes, whose share of a tile is short, read it one tile ahead, so that
+    // its latency hides behind the pair loop; with whole tiles the registers
+    // that this holds cost the loop 2 % instead.
+    constexpr int WJ = SHT > 1 ? SHJ * (TI < 32 ? 32 / TI : 1) : JT;
+    constexpr int WR = WJ / 32;
+    static_assert(WJ % 32 == 0 && (WR <= 2 || WR == NRANGE), "ranges of the warp's j-particles");
+    constexpr bool AHEAD = !FP && TJ > 1;
+    const int wr0 = SHT > 1 ? (tid & ~31) / TI * SHJ / 32 : lane % NRANGE;
+    auto ranges_of = [&](int jt) -> int2 {
+        const int2 *R = a.trange + (size_t)jt * NRANGE + wr0;
+        int2 r = R[0];
+        if constexpr (WR == 2) {
+            const int2 r1 = R[1];
+            r = make_int2(min(r.x, r1.x), max(r.y, r1.y));
+        }
+        return r;
+    };
+    int2 rg_next = make_int2(0, 0);
+    if constexpr (AHEAD)
+        rg_next = ranges_of(jt_next);
     for (int q = 0; q < ntile; ++q) {
-        const long long p = wb + q;
-        while (g_start(cur_g + 1) <= p)
-            ++cur_g;
-        const int t = cur_g;
-        const int jt = jt_of(p, t);
+        if constexpr (!AHEAD) {
+            while (g_start(cur_g + 1) <= wb + q)
+                ++cur_g;
+            jt_next = jt_of(wb + q, cur_g);
+        }
+        const int t = cur_g, jt = jt_next;
+        const int2 rg_tile = rg_next;
+        if (AHEAD && q + 1 < ntile) {
+            while (g_start(cur_g + 1) <= wb + q + 1)
+                ++cur_g;
+            jt_next = jt_of(wb + q + 1, cur_g);
+            rg_next = ranges_of(jt_next);
+        }
         if (t != cur_t) {
             if (cur_t >= 0)
                 finalize(cur_t);
@@ -1073,7 +1118,7 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
         }
         const int s = q % NS;
         const uint32_t par = (uint32_t)((q / NS) & 1);
-        // Does this tile hold the j-particle of one of the warp's i-particles?
+        // Does this range hold the index of one of the warp's i-particles?
         auto self_test = [&](int2 rg) -> bool {
             bool mine = false;
 #pragma unroll
@@ -1090,8 +1135,7 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
             for (int k = 0; k < NI; ++k) {
                 if (tmin[k] < nnr[k]) {
                     nnr[k] = tmin[k];
-                    nnt[k] = jt;
-                    nnc[k] = tchk[k];
+                    nnt[k] = STRIDED ? jt : jt * TJ + tj;
                 }
                 tmin[k] = INF;
             }
@@ -1133,7 +1177,11 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
             pairs_of_tile(pbuf, self_test(rg));
             __syncthreads();                     // pbuf is rewritten by the next tile
         } else {
-            const bool self_tile = self_test(a.trange[jt]);
+            int2 rg = AHEAD ? rg_tile : ranges_of(jt);
+            if constexpr (WR == NRANGE)
+                rg = make_int2(__reduce_min_sync(0xffffffffu, rg.x),
+                               __reduce_max_sync(0xffffffffu, rg.y));
+            const bool self_tile = self_test(rg);
             const bool ready = mbar_wait_bounded(&bar[s], par, a.wait_ns);
             if (!ready)
                 s_abort = 1;
@@ -1495,10 +1543,10 @@ constexpr int fp_smem(int nt, int ni)
 
 const Variant kVariants[] = {
     {{128, 1, 2, 0, G6X_PREC_DS}, k_force_ds<128, 1, 2, false, 3, 2>, 128, ds_smem(128, 2)},
-    {{128, 1, 1, 0, G6X_PREC_DS}, k_force_ds<128, 1, 1, false>, 128, ds_smem(128, 1)},
-    {{64, 4, 1, 0, G6X_PREC_DS}, k_force_ds<64, 4, 1, false>, 256, ds_smem(256, 1)},
-    {{32, 8, 1, 0, G6X_PREC_DS}, k_force_ds<32, 8, 1, false>, 256, ds_smem(256, 1)},
-    {{16, 16, 1, 0, G6X_PREC_DS}, k_force_ds<16, 16, 1, false>, 256, ds_smem(256, 1)},
+    {{128, 1, 1, 0, G6X_PREC_DS}, k_force_ds<128, 1, 1, false, 4>, 128, ds_smem(128, 1)},
+    {{64, 4, 1, 0, G6X_PREC_DS}, k_force_ds<64, 4, 1, false, 2>, 256, ds_smem(256, 1)},
+    {{32, 8, 1, 0, G6X_PREC_DS}, k_force_ds<32, 8, 1, false, 2>, 256, ds_smem(256, 1)},
+    {{16, 16, 1, 0, G6X_PREC_DS}, k_force_ds<16, 16, 1, false, 2>, 256, ds_smem(256, 1)},
     {{128, 1, 1, 1, G6X_PREC_DS}, k_force_ds<128, 1, 1, true>, 128, ds_smem(128, 1)},
     {{32, 1, 1, 1, G6X_PREC_DS}, k_force_ds<32, 1, 1, true>, 32, ds_smem(32, 1)},
     {{128, 1, 1, 0, G6X_PREC_FP64}, k_force_64<false>, 128, 0},
@@ -1515,7 +1563,7 @@ const Variant kVariants[] = {
     {{64, 4, 2, 0, G6X_PREC_DS}, k_force_ds<64, 4, 2, false, 2, 2>, 256, ds_smem(256, 2)},
     // fused prediction (Eq. 1, Eq. 2 inside the force kernel, no separate
     // predictor launch) for small blocks: twins of variants 4, 14, 15, 16
-    {{16, 16, 1, 0, G6X_PREC_DS, 1, 4}, k_force_ds<16, 16, 1, false, 1, 2, false, true>, 256,
+    {{16, 16, 1, 0, G6X_PREC_DS, 1, 4}, k_force_ds<16, 16, 1, false, 2, 2, false, true>, 256,
      fp_smem(256, 1)},
     {{16, 16, 2, 0, G6X_PREC_DS, 1, 14}, k_force_ds<16, 16, 2, false, 2, 2, false, true>, 256,
      fp_smem(256, 2)},
@@ -1526,7 +1574,7 @@ const Variant kVariants[] = {
     // full DS subtraction for the separations (accuracy ablation)
     {{128, 1, 2, 0, G6X_PREC_DS_DSSUB}, k_force_ds<128, 1, 2, false, 3, 2, false, false, true>,
      128, ds_smem(128, 2)},
-    {{16, 16, 1, 0, G6X_PREC_DS_DSSUB}, k_force_ds<16, 16, 1, false, 1, 2, false, false, true>,
+    {{16, 16, 1, 0, G6X_PREC_DS_DSSUB}, k_force_ds<16, 16, 1, false, 2, 2, false, false, true>,
      256, ds_smem(256, 1)},
     // neighbour lists: the twins of variants 9, 4, 14, 15 and 16
     {{128, 1, 2, 1, G6X_PREC_DS}, k_force_ds<128, 1, 2, true, 4, 2>, 128, ds_smem(128, 2)},
@@ -1769,16 +1817,28 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
                       < shapes[k].min_units))
         ++k;
     *gmul = 1;
-    if (shapes[k].v == 9 || shapes[k].v == 23) {
-        // Several waves of CTAs per SM: the warp schedulers favour the
-        // oldest CTAs, so equal shares of the work line finish at different
-        // times, and with one wave the SMs run their last stretch with few
-        // warps.  Later waves fill those slots.  More CTAs also mean more
-        // partial records and i-tile loads, so the count follows the length
-        // of the work line (measured at N = 2^20: 1, 2, 2, 4, 8 waves best
-        // for m = 4096, 16384, 65536, 262144, 2^20).
-        const long long units = (long long)((ni + 255) / 256) * jtl;
+    // Several waves of CTAs per SM: the warp schedulers favour the oldest
+    // CTAs, so equal shares of the work line finish at different times, and
+    // with one wave the SMs run their last stretch with few warps.  Later
+    // waves fill those slots.  More CTAs also mean more partial records and
+    // i-tile loads, so the count follows the length of the work line.
+    const long long units =
+        (long long)((ni + shapes[k].itile - 1) / shapes[k].itile) * jtl;
+    if (shapes[k].v == 23) {
         *gmul = units < (1LL << 18) ? 1 : units < (1LL << 21) ? 2 : units < (1LL << 23) ? 4 : 8;
+    } else if (shapes[k].v == 9) {
+        // measured (force + reduction, ms): 40000 x 131072 (80384 units) 5.53,
+        // 5.46 and 5.45 in 1, 2 and 4 waves; 16384 x 2^20 16.93 in 2, 16.96 in
+        // 8; 65536 x 2^20 67.4, 66.7 and 66.5 in 2, 4 and 8; 4096 x 2^20
+        // (65536 units) 4.39 in 1, 4.38 in 4; 2^18 x 2^20 265.8 in 4, 264.9
+        // in 8; 2^20 x 2^20 1058 in 8
+        *gmul = units <= (1LL << 16) ? 1 : units < (1LL << 19) ? 2
+                : units < (1LL << 21) || units >= (1LL << 23) ? 8 : 4;
+    } else if (shapes[k].v == 16) {
+        // measured (us): 512 x 2^20 (16384 units) 611 in 1 wave, 603 in 2;
+        // 6000 x 131072 896 and 885; 2048 x 2^20 (65536 units) 2345, 2291 and
+        // 2281 in 1, 2 and 4; 384 x 2^20 471 in 1, 474 in 2
+        *gmul = units < (1LL << 14) ? 1 : units < (1LL << 16) ? 2 : 4;
     }
     return shapes[k].v;
 }
