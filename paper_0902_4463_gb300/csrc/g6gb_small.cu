@@ -31,9 +31,8 @@
 //     CTA finishes last.
 //
 // The pair arithmetic and the compensated accumulation are those of K2
-// (k_force_ds); the nearest neighbour is found from the tile still in
-// shared memory whenever a tile lowers a thread's smallest key, instead of
-// K2's rescan of the winning tile from global memory at the end.  Every wait
+// (k_force_ds), and so is the search for the nearest neighbour in the winning
+// share at the end.  Every wait
 // is bounded; a wait that runs out records G6_ETIMEDOUT in the error word and
 // makes the other warps give up at their next wait, and the producer warp
 // keeps the CTA alive until every copy it issued has landed.
@@ -112,6 +111,48 @@ __device__ __forceinline__ PartialDS load_partial_cg(const PartialDS *p)
 
 static_assert(sizeof(PartialDS) == 64, "partial record is four float4");
 
+// Sum of partial records whose nnj is the neighbour's particle index rather
+// than its j-slot, so that the last reduction needs no gather behind it.  The
+// records come in ascending j, so equal distances go to the lower record.
+struct RecordSum : PartialSum<PartialDS> {
+    int ord;                                          // record of the nearest neighbour
+    __device__ void init()
+    {
+        PartialSum<PartialDS>::init();
+        ord = INT_MAX;
+    }
+    __device__ void nearest(float r, int id, int q)
+    {
+        if (id >= 0 && (bj < 0 || r < br || (r == br && q < ord))) {
+            br = r;
+            bj = id;
+            ord = q;
+        }
+    }
+    __device__ void add(const PartialDS &P, int q)
+    {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ds_acc(h[d], l[d], P.acc[d].x, P.acc[d].y);
+            ds_acc(h[3 + d], l[3 + d], P.jerk[d].x, P.jerk[d].y);
+        }
+        ds_acc(h[6], l[6], P.pot.x, P.pot.y);
+        nearest(P.nnr2, P.nnj, q);
+    }
+    __device__ void shfl_combine(int off)
+    {
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+            const float oh = __shfl_xor_sync(0xffffffffu, h[q], off);
+            const float ol = __shfl_xor_sync(0xffffffffu, l[q], off);
+            ds_acc(h[q], l[q], oh, ol);
+        }
+        const float r = __shfl_xor_sync(0xffffffffu, br, off);
+        const int id = __shfl_xor_sync(0xffffffffu, bj, off);
+        nearest(r, id, __shfl_xor_sync(0xffffffffu, ord, off));
+    }
+};
+
 }  // namespace
 
 // TI threads along i x TJ j-groups = 256 compute threads (8 warps, one
@@ -126,8 +167,10 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
     constexpr int ITILE = TI * NI;
     constexpr int PPT = JT / 2 / TJ;                  // j-pairs per thread per tile
     constexpr int FLUSH = (256 + PPT - 1) / PPT;      // tiles between flushes (>= 512 j)
-    constexpr int CHP = PPT < 4 ? PPT : 4;            // j-pairs per neighbour-search chunk
-    static_assert(PPT % CHP == 0, "whole chunks per tile");
+    // j-particles of a tile that a warp walks: the contiguous shares of its
+    // j-groups, one or more of the 32 that one warp predicts
+    constexpr int WJ = JT / TJ * (TI < 32 ? 32 / TI : 1);
+    static_assert(WJ % 32 == 0, "whole predicting warps");
     constexpr int PT_WORDS = JW * JT;                 // one predicted tile
     static_assert(NT == JT, "one j-particle per compute thread when a tile is predicted");
     static_assert(JT % (2 * TJ) == 0, "j-tile must split into j-pairs evenly");
@@ -144,6 +187,7 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
     __shared__ int2 s_wr[2][NW];                      // per predicted tile: each warp's index range
     __shared__ int s_abort, s_last1, s_last2;
     __shared__ float s_ibuf[TJ > 1 ? 11 * ITILE : 1];
+    __shared__ int s_win[TJ > 1 ? ITILE : 1];         // winning share per i-particle
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = gridDim.x, c = blockIdx.x;
@@ -247,7 +291,7 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
     int iid[NI];
     float2 ta[NI][7];
     float tmin[NI], nnr[NI];
-    int nnj[NI], tchk[NI];
+    int nnt[NI];                 // the share (tile x group) with the smallest key
     auto cslot = [&](int k, int q) -> float2 & { return comp[(k * 7 + q) * NT + tid]; };
 #pragma unroll
     for (int k = 0; k < NI; ++k) {
@@ -291,17 +335,22 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
         }
         tmin[k] = INF;
         nnr[k] = INF;
-        nnj[k] = -1;
-        tchk[k] = 0;
+        nnt[k] = -1;
     }
 
     // Eq. 1 and Eq. 2 for tile q (raw stage q % SR) into predicted buffer
     // q & 1, one j-particle per thread; each warp records its index range
     // and hands the raw stage back to the producer.
+    int rstage = 0;                                   // q % SR of the next tile predicted
+    uint32_t rphase = 0;                              // its (q / SR) & 1
     auto predict_into = [&](int q) -> bool {
-        const int r = q % SR, p = q & 1;
-        if (!ws_wait(&rfull[r], (uint32_t)((q / SR) & 1), a.wait_ns, abort_flag, a.err))
+        const int r = rstage, p = q & 1;
+        if (!ws_wait(&rfull[r], rphase, a.wait_ns, abort_flag, a.err))
             return false;
+        if (++rstage == SR) {
+            rstage = 0;
+            rphase ^= 1;
+        }
         const unsigned char *d = raw + (size_t)r * RAW_TILE_BYTES;
         const int jj = tid;
         const int slot = (jb + q) * JT + jj;
@@ -348,25 +397,6 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
             }
     };
 
-    // The key (softened |r|^2, +inf for the i-particle's own j) of j-pair jp
-    // of a predicted tile, with the pair loop's own packed operations.
-    auto pair_key = [&](const float *S, int jp, int k) -> float2 {
-        const float2 xh = reinterpret_cast<const float2 *>(S + W_XH * JT)[jp];
-        const float2 yh = reinterpret_cast<const float2 *>(S + W_YH * JT)[jp];
-        const float2 zh = reinterpret_cast<const float2 *>(S + W_ZH * JT)[jp];
-        const float2 xl = reinterpret_cast<const float2 *>(S + W_XL * JT)[jp];
-        const float2 yl = reinterpret_cast<const float2 *>(S + W_YL * JT)[jp];
-        const float2 zl = reinterpret_cast<const float2 *>(S + W_ZL * JT)[jp];
-        const int2 id = reinterpret_cast<const int2 *>(S + W_ID * JT)[jp];
-        const float2 dx = __fadd2_rn(__fadd2_rn(xh, nxh[k][0]), __fadd2_rn(xl, nxl[k][0]));
-        const float2 dy = __fadd2_rn(__fadd2_rn(yh, nxh[k][1]), __fadd2_rn(yl, nxl[k][1]));
-        const float2 dz = __fadd2_rn(__fadd2_rn(zh, nxh[k][2]), __fadd2_rn(zl, nxl[k][2]));
-        float2 key = soft_r2(dx, dy, dz, eps2);
-        key.x = (id.x == iid[k]) ? INF : key.x;
-        key.y = (id.y == iid[k]) ? INF : key.y;
-        return key;
-    };
-
     // All pairs of the thread's share of one predicted tile (the K2 pair
     // arithmetic, Eq. 3 separations); SELF: with the per-pair self test.
     auto tile_pass = [&](const float *S, auto self_tag) {
@@ -382,10 +412,9 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
         const float2 *VY = reinterpret_cast<const float2 *>(S + W_VY * JT);
         const float2 *VZ = reinterpret_cast<const float2 *>(S + W_VZ * JT);
         const int2 *ID = reinterpret_cast<const int2 *>(S + W_ID * JT);
-        // j-pair kk of the thread's share against its NI i-particles; mins[k]
-        // receives the smaller key
-        auto jpair = [&](int kk, float (&mins)[NI]) {
-            const int jp = tj + kk * TJ;
+        // j-pair kk of the thread's share against its NI i-particles
+        auto jpair = [&](int kk) {
+            const int jp = tj * PPT + kk;
             const float2 xh = XH[jp], yh = YH[jp], zh = ZH[jp], mj = MM[jp];
             const float2 xl = XL[jp], yl = YL[jp], zl = ZL[jp];
             const float2 vx = VX[jp], vy = VY[jp], vz = VZ[jp];
@@ -421,48 +450,37 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
                 ta[k][3] = __ffma2_rn(mr3, __ffma2_rn(sc, dx, ux), ta[k][3]);
                 ta[k][4] = __ffma2_rn(mr3, __ffma2_rn(sc, dy, uy), ta[k][4]);
                 ta[k][5] = __ffma2_rn(mr3, __ffma2_rn(sc, dz, uz), ta[k][5]);
-                mins[k] = fminf(mins[k], fminf(key.x, key.y));
+                tmin[k] = fminf(tmin[k], fminf(key.x, key.y));
             }
         };
-        // by chunks of CHP j-pairs, noting the first chunk that reaches the
-        // tile's minimum, so the neighbour search reads one chunk
-        for (int ch = 0; ch < PPT / CHP; ++ch) {
-            float cm[NI];
-#pragma unroll
-            for (int k = 0; k < NI; ++k)
-                cm[k] = INF;
 #pragma unroll UNR
-            for (int u = 0; u < CHP; ++u)
-                jpair(ch * CHP + u, cm);
-#pragma unroll
-            for (int k = 0; k < NI; ++k)
-                if (cm[k] < tmin[k]) {
-                    tmin[k] = cm[k];
-                    tchk[k] = ch;
-                }
-        }
+        for (int kk = 0; kk < PPT; ++kk)
+            jpair(kk);
     };
 
     // ------------------------------------------------------------ j-tiles
     // Tile q+1 is predicted while tile q's pairs run, into the other buffer;
-    // one barrier per tile then releases both buffers.  Where a tile lowers
-    // an i-particle's smallest key, the first j of the thread's share with
-    // that key is found at once from the tile still in shared memory, in the
-    // chunk the pair loop noted (ties to the lower j-slot: tiles, chunks and
-    // shares are walked in ascending j).
+    // one barrier per tile then releases both buffers.  A thread notes the
+    // tile that lowered an i-particle's smallest key; the neighbour itself is
+    // searched for once, at the end, in the winning share.  (Searching the
+    // tile at once, while still in shared memory, runs in nearly every tile
+    // of a short share of the line, since one lane of the warp is enough:
+    // 3 of the 47 us of m = 16, N = 2^20.)
     bool ok = ntile <= 0 || predict_into(0);
     cta_bar();
     int since_flush = 0;
+    const int wr0 = (warp * 32 / TI) * (JT / TJ) / 32;
     for (int q = 0; q < ntile; ++q) {
         ok = ok && !*abort_flag;
         if (ok && q + 1 < ntile)
             ok = predict_into(q + 1);
         const int p = q & 1;
         if (ok) {
+            // index range of the warp's own j-particles of this tile
             int2 rg = make_int2(INT_MAX, -1);
 #pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                const int2 v = s_wr[p][w];
+            for (int w = 0; w < WJ / 32; ++w) {
+                const int2 v = s_wr[p][wr0 + w];
                 rg.x = min(rg.x, v.x);
                 rg.y = max(rg.y, v.y);
             }
@@ -479,13 +497,7 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
             for (int k = 0; k < NI; ++k) {
                 if (tmin[k] < nnr[k]) {
                     nnr[k] = tmin[k];
-                    for (int kk = tchk[k] * CHP; kk < (tchk[k] + 1) * CHP; ++kk) {
-                        const float2 key = pair_key(S, tj + kk * TJ, k);
-                        if (key.x == nnr[k] || key.y == nnr[k]) {
-                            nnj[k] = (jb + q) * JT + 2 * (tj + kk * TJ) + (key.x == nnr[k] ? 0 : 1);
-                            break;
-                        }
-                    }
+                    nnt[k] = (jb + q) * TJ + tj;
                 }
                 tmin[k] = INF;
             }
@@ -506,6 +518,40 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
     // ------------------------------------------------------------ epilogue
     flush();
     PartialDS *P0 = static_cast<PartialDS *>(a.part);  // [G][ITILE], this CTA's sums
+    // Nearest neighbour of one i-particle in share `share`, by SL lanes
+    // together: from the predicted tile where it is one of the last two, still
+    // in shared memory (always, for a CTA with one or two tiles), else the
+    // share's j-particles predicted again from the j-store.
+    using Search = ShareSearch<TJ>;
+    constexpr int SL = Search::SL;
+    auto nn_scan = [&](int share, const float *xh, const float *xl, int id_i) -> Search {
+        auto key_of = [&](int tile, int jj, int &id) -> float {
+            const int q = tile - jb, slot = tile * JT + jj;
+            float ph[3], pl[3], dd[3];
+            if (q >= ntile - 2) {
+                const float *S = pbuf + (q & 1) * PT_WORDS + jj;
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    ph[d] = S[(W_XH + d) * JT];
+                    pl[d] = S[(W_XL + d) * JT];
+                }
+                id = __float_as_int(S[W_ID * JT]);
+            } else {
+                predict_ds_pos((float)(a.t_pred - js_t0(a.js, slot)), js_xds(a.js, slot),
+                               js_xds2(a.js, slot), js_v0m(a.js, slot), js_a2f(a.js, slot),
+                               js_j6f(a.js, slot), ph, pl);
+                id = js_idx(a.js, slot);
+            }
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                dd[d] = __fadd_rn(__fadd_rn(ph[d], xh[d]), __fadd_rn(pl[d], xl[d]));
+            const float key = soft_r2(dd[0], dd[1], dd[2], eps2.x);
+            return id == id_i ? INF : key;
+        };
+        Search w;
+        w.scan(share, key_of);
+        return w;
+    };
     if constexpr (TJ > 1) {
         // The TJ j-groups of an i-particle combine in compensated FP32,
         // nearest neighbour ties to the lower j-slot.  First inside each warp:
@@ -533,7 +579,7 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
                 l[q] = hl.y;
             }
             float br = nnr[k];
-            int bj = nnj[k];
+            int bj = nnt[k];
 #pragma unroll
             for (int off = TIW; off < 32; off <<= 1) {
 #pragma unroll
@@ -589,7 +635,32 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
             }
             P->pot = make_float2(sh[6], sl[6]);
             P->nnr2 = unsoftened(br, eps2.x);
-            P->nnj = bj;
+            s_win[il] = bj;
+        }
+        cta_bar();
+        static_assert(ITILE % (32 / SL) == 0, "whole warps search together");
+        constexpr int SPR = NT / SL;                  // i-particles searched per round
+        constexpr int SW = ITILE > 2 * SPR ? 4 : ITILE > SPR ? 2 : 1;   // rounds in flight
+        for (int i0 = tid / SL; i0 < ITILE; i0 += SW * SPR) {
+            Search w[SW];
+#pragma unroll
+            for (int r = 0; r < SW; ++r) {
+                const int il = i0 + r * SPR, is = il < ITILE ? il : i0;
+                float xh[3], xl[3];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    xh[d] = -s_ibuf[d * ITILE + is];
+                    xl[d] = -s_ibuf[(3 + d) * ITILE + is];
+                }
+                w[r] = nn_scan(il < a.ni ? s_win[is] : -1, xh, xl,
+                               __float_as_int(s_ibuf[10 * ITILE + is]));
+            }
+#pragma unroll
+            for (int r = 0; r < SW; ++r) {
+                const int il = i0 + r * SPR, id = w[r].template agree<true>();
+                if (lane % SL == 0 && il < ITILE)
+                    P0[(size_t)c * ITILE + il].nnj = id;
+            }
         }
     } else {
 #pragma unroll
@@ -602,7 +673,22 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
             }
             P->pot = cslot(k, 6);
             P->nnr2 = unsoftened(nnr[k], eps2.x);
-            P->nnj = nnj[k];
+            // each of the warp's i-particles in turn, by the whole warp
+            int nnj = -1;
+            for (int l = 0; l < 32; ++l) {
+                float xh[3], xl[3];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    xh[d] = __shfl_sync(0xffffffffu, nxh[k][d].x, l);
+                    xl[d] = __shfl_sync(0xffffffffu, nxl[k][d].x, l);
+                }
+                const int id = nn_scan(__shfl_sync(0xffffffffu, nnt[k], l), xh, xl,
+                                       __shfl_sync(0xffffffffu, iid[k], l))
+                                   .template agree<true>();
+                if (lane == l)
+                    nnj = id;
+            }
+            P->nnj = nnj;
         }
     }
 
@@ -619,12 +705,19 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
         const int part = tid % P;
         for (int rr = 0; rr < rounds; ++rr) {
             const int il = rr * groups + tid / P;
-            PartialSum<PartialDS> acc;
+            RecordSum acc;
             acc.init();
             if (il < ITILE) {
-#pragma unroll 4
-                for (int q = part; q < nrec; q += P)
-                    acc.add(load_partial_cg(src + (size_t)q * ITILE + il));
+                // two records of a lane in flight at once
+                for (int q = part; q < nrec; q += 2 * P) {
+                    const bool two = q + P < nrec;
+                    const PartialDS r0 = load_partial_cg(src + (size_t)q * ITILE + il);
+                    const PartialDS r1 =
+                        load_partial_cg(src + (size_t)(two ? q + P : q) * ITILE + il);
+                    acc.add(r0, q);
+                    if (two)
+                        acc.add(r1, q + P);
+                }
             }
             for (int off = P / 2; off > 0; off >>= 1)
                 acc.shfl_combine(off);
@@ -640,7 +733,17 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
                     D->nnr2 = acc.br;
                     D->nnj = acc.bj;
                 } else if (il < a.ni) {
-                    a.out[il] = result_of(acc, a.jidx);
+                    g6x_out o;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        o.acc[d] = acc.value(d);
+                        o.jerk[d] = acc.value(3 + d);
+                    }
+                    o.pot = -acc.value(6);
+                    const bool has_nn = acc.bj >= 0 && acc.nnr2() < 1e30f;
+                    o.nnb = has_nn ? acc.bj : -1;
+                    o.nnr2 = has_nn ? acc.nnr2() : INF;
+                    a.out[il] = o;
                 }
             }
         }
@@ -701,11 +804,11 @@ constexpr int ws_smem(int sr, int ni)
 
 // VariantInfo: ti, tj, nper, list, prec, fpred, twin, ws
 const WsVariant kWs[] = {
-    {{16, 16, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 1, 2, 3>, ws_smem(3, 1)},
-    {{32, 8, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 1, 2, 3>, ws_smem(3, 1)},
-    {{64, 4, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<64, 4, 1, 2, 3>, ws_smem(3, 1)},
-    {{128, 2, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<128, 2, 1, 2, 3>, ws_smem(3, 1)},
-    {{256, 1, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<256, 1, 1, 2, 3>, ws_smem(3, 1)},
+    {{16, 16, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 1, 2, 3, 4>, ws_smem(3, 1)},
+    {{32, 8, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 1, 2, 3, 4>, ws_smem(3, 1)},
+    {{64, 4, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<64, 4, 1, 2, 3, 4>, ws_smem(3, 1)},
+    {{128, 2, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<128, 2, 1, 2, 3, 4>, ws_smem(3, 1)},
+    {{256, 1, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<256, 1, 1, 2, 3, 4>, ws_smem(3, 1)},
     // two i-particles per thread, one CTA per SM with a deeper ring
     {{16, 16, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 2, 1, 6>, ws_smem(6, 2)},
     {{32, 8, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 2, 1, 6>, ws_smem(6, 2)},
@@ -718,6 +821,11 @@ constexpr int kNumWs = (int)(sizeof(kWs) / sizeof(kWs[0]));
 int g_ws_occ[kNumWs];
 
 }  // namespace
+
+// Grids of up to this many CTAs reduce in one level: the second level costs
+// an arrival, a fence and a round of loads (2.5 of the 14.3 us of a block
+// step at N = 1024, 4 CTAs) that a few more records per lane do not.
+constexpr int WS_ONE_LEVEL = 32;
 
 int ws_variant_count() { return kNumWs; }
 
@@ -755,6 +863,9 @@ int ws_variant_occupancy(int k)
 
 int ws_group_size(int grid)
 {
+    // one level while the last CTA's lanes hold a few records each
+    if (grid <= WS_ONE_LEVEL)
+        return grid;
     int gs = 1;
     while (gs * gs < grid)
         ++gs;
