@@ -37,6 +37,7 @@ namespace {
 
 constexpr int NSTAGE = 3;
 constexpr int FP_NSTAGE = 2;        // raw-tile stages of the fused-prediction kernels
+constexpr int JS64 = 64;            // j-particles per sub-tile of the FP64 kernel
 
 }  // namespace
 
@@ -1199,84 +1200,156 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
     finalize(cur_t);
 }
 
-// The same pair sum entirely in FP64, one i-particle per thread, j-tiles
-// staged in shared memory by plain cooperative loads.
-template <bool LIST>
+// 1 / sqrt(s) in FP64: the hardware's approximation refined by one step of
+// Householder's third-order iteration (A. S. Householder, The Numerical
+// Treatment of a Single Nonlinear Equation, 1970): with e = 1 - s y0^2,
+// y = y0 + y0 e (1/2 + 3/8 e) leaves 5/16 e^3, below a rounding for an
+// approximation good to 2^-20.  Five FP64 operations.  Zero, infinity and
+// subnormal s take the library's function.
+__device__ __forceinline__ double rsqrt64(double s)
+{
+    const unsigned hi = (unsigned)__double2hiint(s);
+    if (hi - 0x00100000u >= 0x7fe00000u)
+        return rsqrt(s);
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(s));
+    const double e = fma(-(s * y0), y0, 1.0);
+    return fma(y0 * e, fma(0.375, e, 0.5), y0);
+}
+
+// The same pair sum entirely in FP64, one i-particle per thread: TI threads
+// along i x TJ j-groups of 128 threads, sub-tiles of JS j-particles staged in
+// shared memory by plain cooperative loads, one ahead in registers.
+//
+// Bound by the FP64 pipe (2 lanes per clock and SM): 33 FP64 operations per
+// pair, and nothing else on that pipe: the neighbour and list tests compare
+// the keys as unsigned integers (they are not negative, so the order is the
+// same; a NaN of either sign still loses) and the index as bits.  With one i-particle per thread of
+// 128 and tiles of 256 a block of 793 paid for 896 lanes and CTAs of one unit
+// each; 32-wide i-tiles pay for 800, and the line of 64-wide sub-tiles is cut
+// evenly over the SMs.  Force alone, before and after (us): m = 793, N =
+// 32768: 1941 and 1588; m = 972, N = 131072: 9776 and 7686 (0.79 of the pipe at
+// 60 operations per pair); m = 32, N = 32768: 340 and 84; m = 1 (8-wide
+// i-tiles): 338 and 32; m = 7, N = 1024: 336 and 16.
+template <int TJ, bool LIST>
 __global__ void __launch_bounds__(128) k_force_64(const ForceArgs a)
 {
     grid_dep_wait();                // the FP64 prediction (see k_force_ds)
     grid_dep_launch();
-    constexpr int TI = 128;
-    __shared__ double4_32a sp[JT], sv[JT];
-    const int tid = threadIdx.x;
+    constexpr int NT = 128, TI = NT / TJ, SH = JS64 / TJ;
+    static_assert(TJ == 1 || !LIST, "lists: whole sub-tiles per thread (ascending j)");
+    static_assert(SH >= 1 && 2 * JS64 == NT, "one record per thread and sub-tile");
+    __shared__ double4_32a sj[2][2][JS64];            // two sub-tiles: (x, m), (v, index)
+    __shared__ double s_sum[TJ > 1 ? 7 * NT : 1];
+    __shared__ unsigned long long s_key[TJ > 1 ? NT : 1];
+    __shared__ int s_nnj[TJ > 1 ? NT : 1];
+    const int tid = threadIdx.x, ti = tid % TI, tj = TJ > 1 ? tid / TI : 0;
     const long long G = gridDim.x, c = blockIdx.x;
     const long long wb = work_begin(c, a.W, G), we = work_begin(c + 1, a.W, G);
     if (we <= wb)
         return;
-    double xi[3] = {0, 0, 0}, vi[3] = {0, 0, 0}, h2 = 0.0;
-    int iid = -2;
+    double xi[3] = {0, 0, 0}, vi[3] = {0, 0, 0};
+    unsigned long long h2 = 0;                        // the radius' bits; 0: no list
+    double idx = -2.0;                                // the index as the j-records carry it
     double s[7];
-    double nnr = 0.0;
+    constexpr unsigned long long INF = 0x7ff0000000000000ull;
+    unsigned long long nnr = INF;
     int nnj = -1, nbn = 0;
-    int cur_t = -1;
-    const double INF = __longlong_as_double(0x7ff0000000000000ll);
 
     auto finalize = [&](int t) {
         const long long seg = c + t;
-        Partial64 *P = reinterpret_cast<Partial64 *>(a.part) + (size_t)seg * TI + tid;
-        for (int d = 0; d < 3; ++d) {
-            P->acc[d] = s[d];
-            P->jerk[d] = s[3 + d];
+        if constexpr (TJ > 1) {
+#pragma unroll
+            for (int q = 0; q < 7; ++q)
+                s_sum[q * NT + tid] = s[q];
+            s_key[tid] = nnr;
+            s_nnj[tid] = nnj;
+            __syncthreads();
+            if (tid < TI) {
+#pragma unroll
+                for (int g = 1; g < TJ; ++g) {
+                    const int o = g * TI + tid;
+#pragma unroll
+                    for (int q = 0; q < 7; ++q)
+                        s[q] += s_sum[q * NT + o];
+                    const unsigned long long k = s_key[o];
+                    const int j = s_nnj[o];
+                    if (j >= 0 && (nnj < 0 || k < nnr || (k == nnr && j < nnj))) {
+                        nnr = k;
+                        nnj = j;
+                    }
+                }
+            }
         }
-        P->pot = s[6];
-        P->nnr2 = nnr;
-        P->nnj = nnj;
-        if constexpr (LIST) {
-            a.nbc[(size_t)seg * TI + tid] = nbn;
-            if (nbn > 0)
-                atomicMax(a.nbmax, min(nbn, a.maxnb));
+        if (TJ == 1 || tid < TI) {
+            Partial64 *P = reinterpret_cast<Partial64 *>(a.part) + (size_t)seg * TI + ti;
+            for (int d = 0; d < 3; ++d) {
+                P->acc[d] = s[d];
+                P->jerk[d] = s[3 + d];
+            }
+            P->pot = s[6];
+            P->nnr2 = __longlong_as_double((long long)nnr);
+            P->nnj = nnj;
+            if constexpr (LIST) {
+                a.nbc[(size_t)seg * TI + ti] = nbn;
+                if (nbn > 0)
+                    atomicMax(a.nbmax, min(nbn, a.maxnb));
+            }
         }
     };
 
+    // this thread's record of a sub-tile: the first JS64 threads the
+    // positions, the others the velocities
+    const double4_32a *src = tid < JS64 ? a.p64 + tid : a.v64 + (tid - JS64);
+    int t = (int)(wb / a.J), jt = (int)(wb - (long long)t * a.J), cur_t = -1;
+    double4_32a next = src[(size_t)jt * JS64];
     for (long long p = wb; p < we; ++p) {
-        const int t = (int)(p / a.J);
-        const int jt = (int)(p - (long long)t * a.J);
-        if (t != cur_t) {
+        const int b = (int)((p - wb) & 1);
+        sj[b][tid >= JS64][tid & (JS64 - 1)] = next;
+        const int t_now = t, jbase = jt * JS64;
+        if (++jt == a.J) {
+            jt = 0;
+            ++t;
+        }
+        if (p + 1 < we)
+            next = src[(size_t)jt * JS64];
+        if (t_now != cur_t) {
             if (cur_t >= 0)
                 finalize(cur_t);
-            long long gi = (long long)t * TI + tid;
+            const long long gi = (long long)t_now * TI + ti;
             if (gi < a.ni) {
                 const g6x_irec &r = a.irec[gi];
                 for (int d = 0; d < 3; ++d) {
                     xi[d] = r.x[d];
                     vi[d] = r.v[d];
                 }
-                h2 = r.h2;
-                iid = r.index;
+                h2 = r.h2 > 0.0 ? (unsigned long long)__double_as_longlong(r.h2) : 0;
+                idx = (double)r.index;
             } else {
-                iid = -2;
+                h2 = 0;
+                idx = -2.0;
             }
             for (int q = 0; q < 7; ++q)
                 s[q] = 0.0;
             nnr = INF;
             nnj = -1;
             nbn = 0;
-            cur_t = t;
+            cur_t = t_now;
         }
+        // the buffer of the sub-tile before is written again only after the
+        // next barrier, which every thread reaches behind its pair loop
         __syncthreads();
-        for (int k = tid; k < JT; k += TI) {
-            sp[k] = a.p64[(size_t)jt * JT + k];
-            sv[k] = a.v64[(size_t)jt * JT + k];
-        }
-        __syncthreads();
-        const int jbase = jt * JT;
-        for (int jj = 0; jj < JT; ++jj) {
-            const double4_32a pj = sp[jj], vj = sv[jj];
+        const long long id_i = __double_as_longlong(idx);
+#pragma unroll 2
+        for (int jj = 0; jj < SH; ++jj) {
+            const double4_32a pj = sj[b][0][tj * SH + jj], vj = sj[b][1][tj * SH + jj];
             const double dx = pj.x - xi[0], dy = pj.y - xi[1], dz = pj.z - xi[2];
             const double ux = vj.x - vi[0], uy = vj.y - vi[1], uz = vj.z - vi[2];
             const double r2u = dx * dx + dy * dy + dz * dz;
-            const double key = ((int)vj.w == iid) ? INF : r2u;
-            const double ri = rsqrt(key + a.eps2);
+            const unsigned long long key =
+                __double_as_longlong(vj.w) == id_i ? INF
+                                                   : (unsigned long long)__double_as_longlong(r2u);
+            const double ri = rsqrt64(__longlong_as_double((long long)key) + a.eps2);
             const double rv = dx * ux + dy * uy + dz * uz;
             const double ri2 = ri * ri;
             const double mr = pj.w * ri;
@@ -1291,12 +1364,12 @@ __global__ void __launch_bounds__(128) k_force_64(const ForceArgs a)
             s[5] += mr3 * (uz + sc * dz);
             if (key < nnr) {
                 nnr = key;
-                nnj = jbase + jj;
+                nnj = jbase + tj * SH + jj;
             }
             if constexpr (LIST) {
                 if (key < h2) {
                     if (nbn < a.nbseg)
-                        a.nbl[((size_t)(c + t) * TI + tid) * a.nbseg + nbn] = jbase + jj;
+                        a.nbl[((size_t)(c + t_now) * TI + ti) * a.nbseg + nbn] = jbase + jj;
                     ++nbn;
                 }
             }
@@ -1549,8 +1622,8 @@ const Variant kVariants[] = {
     {{16, 16, 1, 0, G6X_PREC_DS}, k_force_ds<16, 16, 1, false, 2>, 256, ds_smem(256, 1)},
     {{128, 1, 1, 1, G6X_PREC_DS}, k_force_ds<128, 1, 1, true>, 128, ds_smem(128, 1)},
     {{32, 1, 1, 1, G6X_PREC_DS}, k_force_ds<32, 1, 1, true>, 32, ds_smem(32, 1)},
-    {{128, 1, 1, 0, G6X_PREC_FP64}, k_force_64<false>, 128, 0},
-    {{128, 1, 1, 1, G6X_PREC_FP64}, k_force_64<true>, 128, 0},
+    {{32, 4, 1, 0, G6X_PREC_FP64}, k_force_64<4, false>, 128, 0},
+    {{128, 1, 1, 1, G6X_PREC_FP64}, k_force_64<1, true>, 128, 0},
     // alternative shapes, for tuning
     {{128, 1, 2, 0, G6X_PREC_DS}, k_force_ds<128, 1, 2, false, 4, 2>, 128, ds_smem(128, 2)},
     {{128, 1, 2, 0, G6X_PREC_DS}, k_force_ds<128, 1, 2, false, 3, 4>, 128, ds_smem(128, 2)},
@@ -1582,6 +1655,9 @@ const Variant kVariants[] = {
     {{16, 16, 2, 1, G6X_PREC_DS}, k_force_ds<16, 16, 2, true, 2, 2>, 256, ds_smem(256, 2)},
     {{32, 8, 2, 1, G6X_PREC_DS}, k_force_ds<32, 8, 2, true, 2, 2>, 256, ds_smem(256, 2)},
     {{64, 4, 2, 1, G6X_PREC_DS}, k_force_ds<64, 4, 2, true, 2, 2>, 256, ds_smem(256, 2)},
+    // FP64, narrow i-tiles
+    {{16, 8, 1, 0, G6X_PREC_FP64}, k_force_64<8, false>, 128, 0},
+    {{8, 16, 1, 0, G6X_PREC_FP64}, k_force_64<16, false>, 128, 0},
 };
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 
@@ -1755,8 +1831,21 @@ constexpr long long WS_MIN_JTILES = 2048;
 int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int *gmul)
 {
     *gmul = 1;
-    if (prec == G6X_PREC_FP64)
-        return list ? 8 : 7;
+    if (prec == G6X_PREC_FP64) {
+        if (list)
+            return 8;
+        // the FP64 pipe pays for every lane, so the i-tile that pads the
+        // block least (ties to the widest; large blocks pad little either way)
+        static constexpr int shapes64[] = {7, 28, 29};
+        int best = 7;
+        if (ni <= 256)
+            for (int v : shapes64) {
+                const int w = kVariants[v].info.ti, u = kVariants[best].info.ti;
+                if ((ni + w - 1) / w * w < (ni + u - 1) / u * u)
+                    best = v;
+            }
+        return best;
+    }
     if (prec == G6X_PREC_DS_DSSUB && !list) {
         *gmul = ni > 2048 ? 2 : 1;
         return ni <= 32 ? 22 : 21;
@@ -1849,6 +1938,9 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
 // kernel (where the caller allows a fused prediction).
 bool g_ws_default = true;
 
+// The FP64 kernel cuts its work line in sub-tiles of JS64 j-particles.
+static int subtiles(int prec) { return prec == G6X_PREC_FP64 ? JT / JS64 : 1; }
+
 ForceConfig choose_config(int prec, int ni, int nj_pad, int list, int sm_count,
                           int force_variant, int force_grid, bool allow_fpred)
 {
@@ -1894,8 +1986,8 @@ ForceConfig choose_config(int prec, int ni, int nj_pad, int list, int sm_count,
     if (occ < 1)
         occ = 1;
     long long g = force_grid > 0 ? force_grid : (long long)sm_count * occ * gmul;
-    if (g > c.work)
-        g = c.work;
+    if (g > c.work * subtiles(c.prec))
+        g = c.work * subtiles(c.prec);
     if (g < 1)
         g = 1;
     c.grid = (int)g;
@@ -2035,8 +2127,8 @@ cudaError_t launch_force(const ForceConfig &cfg, const Pred &p,
     if (cfg.list && cfg.tj > 1)
         a.nbr = nbl_part + partial_slots(cfg) * (size_t)lists->nbseg;
     a.err = d_err;
-    a.W = cfg.work;
-    a.J = cfg.jtiles;
+    a.W = cfg.work * subtiles(cfg.prec);
+    a.J = cfg.jtiles * subtiles(cfg.prec);
     a.ni = ni;
     a.eps2 = eps2;
     a.wait_ns = g_wait_ns;
@@ -2114,8 +2206,8 @@ cudaError_t launch_reduce(const ForceConfig &cfg, const void *part,
     a.out = d_out;
     a.nbl_out = d_nbl;
     a.nblen_out = d_nblen;
-    a.W = cfg.work;
-    a.J = cfg.jtiles;
+    a.W = cfg.work * subtiles(cfg.prec);
+    a.J = cfg.jtiles * subtiles(cfg.prec);
     a.G = cfg.grid;
     a.ni = ni;
     a.itile = cfg.itile;
