@@ -657,12 +657,41 @@ ForceConfig pick_config(const Ctx &c, int nj, int ni, bool list)
 // j-store update, prediction (unless the force kernel predicts itself),
 // force and reduction.
 int run_force(Ctx &c, const ForceConfig &cfg, int nj, int ni, const g6x_irec *d_irec,
-              double eps2, g6x_out *d_out, bool folded);
+              double eps2, g6x_out *d_out, bool folded, const g6::WsInline *in = nullptr);
 
+// Whether the records of a block step fit the arguments of its one launch:
+// few of them, the staged j-records all in the j-tiles that the launch reads.
+bool fits_inline(const Ctx &c, const ForceConfig &cfg, int ni)
+{
+    if (ni > g6::WS_INLINE || c.n_jst > g6::WS_INLINE || !g6::ws_takes_inline(cfg))
+        return false;
+    for (int k = 0; k < c.n_jst; ++k)
+        if (c.h_jst[k].address / JT >= cfg.jtiles)
+            return false;
+    return true;
+}
+
+// h_irec: the i-records in host memory, where they are there (else NULL).
 int predict_and_force(Ctx &c, int nj, int ni, const g6x_irec *d_irec, double eps2, bool list,
-                      g6x_out *d_out)
+                      g6x_out *d_out, const g6x_irec *h_irec = nullptr)
 {
     const ForceConfig cfg = pick_config(c, nj, ni, list);
+    if (h_irec && ni > 0 && fits_inline(c, cfg, ni)) {
+        // a few particles: the launch carries their records, so nothing is
+        // sorted or read back over the host link
+        g6::WsInline in;
+        in.nrec = c.n_jst;
+        std::memcpy(in.rec, c.h_jst, sizeof(g6x_jrec) * c.n_jst);
+        std::memcpy(in.irec, h_irec, sizeof(g6x_irec) * ni);
+        const int rc = run_force(c, cfg, nj, ni, d_irec, eps2, d_out, false, &in);
+        if (!rc && c.n_jst) {
+            for (int k = 0; k < c.n_jst; ++k)
+                c.slot_of[c.h_jst[k].address] = -1;
+            c.n_jst = 0;
+            c.ver += 1;            // the cached predictions are stale
+        }
+        return rc;
+    }
     const bool fp = g6::variant_info(cfg.variant).fpred != 0 && ni > 0;
     // a small block is one launch: the fused-prediction kernel also stores
     // the staged records of its tiles
@@ -710,7 +739,7 @@ int ensure_counters(Ctx &c, size_t n)
 }
 
 int run_force(Ctx &c, const ForceConfig &cfg, int nj, int ni, const g6x_irec *d_irec,
-              double eps2, g6x_out *d_out, bool folded)
+              double eps2, g6x_out *d_out, bool folded, const g6::WsInline *in)
 {
     // fused-prediction shapes read the j-store itself (the predicted tiles
     // and their cache entry are left as they are); folded: they also store
@@ -759,7 +788,7 @@ int run_force(Ctx &c, const ForceConfig &cfg, int nj, int ni, const g6x_irec *d_
             return rc;
         PhaseTimer pt(c, PH_FORCE);
         e = g6::launch_force_ws(cfg, d_irec, ni, eps2, nj, c.d_part, c.d_tcnt, d_out, c.js.idx,
-                                c.d_err, fpa, c.stream, pdl);
+                                c.d_err, fpa, c.stream, pdl, in);
         c.launches += 1;
     } else if (cfg.prec == G6X_PREC_DS && seg_per_tile <= g6::FUSED_MAX_SEGS) {
         // one launch: the last CTA of each i-tile reduces it (K3 fused into
@@ -1100,7 +1129,7 @@ void g6calc_firsthalf(int cid, int nj, int ni, const int index[],
     // the kernels read the i-records from, and write results to, the mapped
     // host buffers: no separate copies
     if (!rc)
-        rc = predict_and_force(*c, nj, ni, c->d_irec, eps2, list, c->d_out);
+        rc = predict_and_force(*c, nj, ni, c->d_irec, eps2, list, c->d_out, c->h_irec);
     if (!rc && ni > 0) {
         if (!rc && h2 && !list) {
             // every radius is <= 0: no list can have entries; skip the list

@@ -123,6 +123,15 @@ struct VariantInfo {
                        // reduced inside the launch (two levels)
 };
 
+// The records of a small block step as arguments of its launch: staged
+// j-records (in any order) and i-records.
+constexpr int WS_INLINE = 32;
+struct WsInline {
+    int nrec = 0;
+    g6x_jrec rec[WS_INLINE];
+    g6x_irec irec[WS_INLINE];
+};
+
 // What a fused-prediction force kernel needs: the raw j-store, the block
 // time and the number of particles in j-memory (DS + SP predictor only).
 struct FusedPred {
@@ -282,7 +291,11 @@ cudaError_t launch_force_fused(const ForceConfig &cfg, const Pred &p,
 // counters, zero before the launch and left zero by a launch that completes.
 cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int ni, double eps2,
                             int nj, void *part, unsigned *cnt, g6x_out *out, const int *jidx,
-                            int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl);
+                            int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl,
+                            const WsInline *in = nullptr);
+// Whether launch_force_ws takes this launch's records from `in` (i-tiles of
+// up to WS_INLINE; then d_irec, fp.rec and fp.toff are not read).
+bool ws_takes_inline(const ForceConfig &cfg);
 cudaError_t launch_reduce(const ForceConfig &cfg, const void *part,
                           const int *nbl_part, const int *nbc_part,
                           const int *jidx, int ni, g6x_out *d_out,

@@ -111,6 +111,19 @@ __device__ __forceinline__ PartialDS load_partial_cg(const PartialDS *p)
 
 static_assert(sizeof(PartialDS) == 64, "partial record is four float4");
 
+// No records in the launch's arguments.
+struct WsNone {
+};
+// i-record il: from the launch's arguments, or from device memory.
+__device__ __forceinline__ const g6x_irec &irec_of(const ForceArgs &, int il, const WsInline &in)
+{
+    return in.irec[il];
+}
+__device__ __forceinline__ const g6x_irec &irec_of(const ForceArgs &a, int il, const WsNone &)
+{
+    return a.irec[il];
+}
+
 // Sum of partial records whose nnj is the neighbour's particle index rather
 // than its j-slot, so that the last reduction needs no gather behind it.  The
 // records come in ascending j, so equal distances go to the lower record.
@@ -159,9 +172,17 @@ struct RecordSum : PartialSum<PartialDS> {
 // j-particle each when a tile is predicted), NI i-particles per thread, so
 // the i-tile is TI x NI; one producer warp; MINB CTAs per SM; SR raw stages;
 // UNR j-pairs of the pair loop unrolled together.
-template <int TI, int TJ, int NI, int MINB, int SR, int UNR = 2>
-__global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs a)
+//
+// IN: the block's staged j-records and i-records come as arguments of the
+// launch (WsInline) instead of from mapped host memory, where each CTA waits
+// for a chain of reads over the host link (the range of its tiles' records,
+// the records, then the copy that may read them) before its first tile.
+template <int TI, int TJ, int NI, int MINB, int SR, int UNR, class IN>
+__global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs a, const __grid_constant__ IN in)
 {
+    constexpr bool INLINE = std::is_same<IN, WsInline>::value;
+    static_assert(!INLINE || (TJ > 1 && TI * NI <= WS_INLINE),
+                  "records in the arguments: narrow i-tiles");
     constexpr int NT = TI * TJ;                       // compute threads
     constexpr int NW = NT / 32;                       // compute warps
     constexpr int ITILE = TI * NI;
@@ -208,9 +229,22 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
                  &rfull[s]);
     };
     if (warp == NW) {
-        // the staged j-records of this CTA's tiles (sorted by tile, so one
-        // contiguous range), stored before any copy reads the tiles
-        if (a.rec && ntile > 0) {
+        // the staged j-records of this CTA's tiles (in the arguments, or sorted
+        // by tile, so one contiguous range), stored before any copy reads the
+        // tiles
+        if constexpr (INLINE) {
+            bool any = false;
+            for (int r = lane; r < in.nrec; r += 32) {
+                const int q = in.rec[r].address / JT - jb;
+                if (q >= 0 && q < ntile) {
+                    store_record(in.rec[r], a.js);
+                    any = true;
+                }
+            }
+            if (__any_sync(0xffffffffu, any))
+                fence_proxy_async_global();
+            __syncwarp();
+        } else if (a.rec && ntile > 0) {
             const int r0 = a.toff[jb], r1 = a.toff[jb + ntile];
             for (int r = r0 + lane; r < r1; r += 32)
                 store_record(a.rec[r], a.js);
@@ -233,7 +267,7 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
             for (int il = tid; il < ITILE; il += NT) {
                 float w[11];
                 if (il < a.ni) {
-                    const g6x_irec &r = a.irec[il];
+                    const g6x_irec &r = irec_of(a, il, in);
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const double x = r.x[d];
@@ -787,12 +821,14 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
 
 namespace {
 
-using WsFn = void (*)(const ForceArgs);
+using WsFn = void (*)(const ForceArgs, const WsNone);
+using WsInFn = void (*)(const ForceArgs, const WsInline);
 
 struct WsVariant {
     VariantInfo info;
     WsFn fn;
     int smem;
+    WsInFn fn_in = nullptr;        // the same with the records in the arguments
 };
 
 // dynamic shared memory: SR raw stages, two predicted tiles, the
@@ -804,18 +840,21 @@ constexpr int ws_smem(int sr, int ni)
 
 // VariantInfo: ti, tj, nper, list, prec, fpred, twin, ws
 const WsVariant kWs[] = {
-    {{16, 16, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 1, 2, 3, 4>, ws_smem(3, 1)},
-    {{32, 8, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 1, 2, 3, 4>, ws_smem(3, 1)},
-    {{64, 4, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<64, 4, 1, 2, 3, 4>, ws_smem(3, 1)},
-    {{128, 2, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<128, 2, 1, 2, 3, 4>, ws_smem(3, 1)},
-    {{256, 1, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<256, 1, 1, 2, 3, 4>, ws_smem(3, 1)},
+    {{16, 16, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 1, 2, 3, 4, WsNone>, ws_smem(3, 1),
+     k_force_ws<16, 16, 1, 2, 3, 4, WsInline>},
+    {{32, 8, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 1, 2, 3, 4, WsNone>, ws_smem(3, 1),
+     k_force_ws<32, 8, 1, 2, 3, 4, WsInline>},
+    {{64, 4, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<64, 4, 1, 2, 3, 4, WsNone>, ws_smem(3, 1)},
+    {{128, 2, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<128, 2, 1, 2, 3, 4, WsNone>, ws_smem(3, 1)},
+    {{256, 1, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<256, 1, 1, 2, 3, 4, WsNone>, ws_smem(3, 1)},
     // two i-particles per thread, one CTA per SM with a deeper ring
-    {{16, 16, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 2, 1, 6>, ws_smem(6, 2)},
-    {{32, 8, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 2, 1, 6>, ws_smem(6, 2)},
-    {{64, 4, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<64, 4, 2, 1, 6>, ws_smem(6, 2)},
-    {{128, 2, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<128, 2, 2, 1, 6>, ws_smem(6, 2)},
+    {{16, 16, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<16, 16, 2, 1, 6, 2, WsNone>, ws_smem(6, 2)},
+    {{32, 8, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<32, 8, 2, 1, 6, 2, WsNone>, ws_smem(6, 2)},
+    {{64, 4, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<64, 4, 2, 1, 6, 2, WsNone>, ws_smem(6, 2)},
+    {{128, 2, 2, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<128, 2, 2, 1, 6, 2, WsNone>, ws_smem(6, 2)},
     // the narrowest i-tile, for blocks of up to 8
-    {{8, 32, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<8, 32, 1, 2, 3>, ws_smem(3, 1)},
+    {{8, 32, 1, 0, G6X_PREC_DS, 1, -1, 1}, k_force_ws<8, 32, 1, 2, 3, 2, WsNone>, ws_smem(3, 1),
+     k_force_ws<8, 32, 1, 2, 3, 2, WsInline>},
 };
 constexpr int kNumWs = (int)(sizeof(kWs) / sizeof(kWs[0]));
 int g_ws_occ[kNumWs];
@@ -850,6 +889,17 @@ int ws_variant_occupancy(int k)
                              cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
         cudaGetLastError();
+        if (v.fn_in) {
+            if (cudaFuncSetAttribute(v.fn_in, cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem)
+                != cudaSuccess) {
+                cudaGetLastError();
+                return 0;
+            }
+            cudaFuncSetAttribute(reinterpret_cast<const void *>(v.fn_in),
+                                 cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+            cudaGetLastError();
+        }
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, v.fn, JT + 32, v.smem)
             != cudaSuccess) {
@@ -880,7 +930,8 @@ size_t ws_partial_slots(int grid, int itile)
 
 cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int ni, double eps2,
                             int nj, void *part, unsigned *cnt, g6x_out *out, const int *jidx,
-                            int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl)
+                            int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl,
+                            const WsInline *in)
 {
     const int k = cfg.variant - (variant_count() - kNumWs);
     const int grid = cfg.grid, jtiles = cfg.jtiles;
@@ -908,7 +959,18 @@ cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int 
     a.toff = fp.toff;
     a.gs = ws_group_size(grid);
     const WsVariant &v = kWs[k];
-    return launch_maybe_pdl(v.fn, grid, JT + 32, v.smem, s, pdl, a);
+    if (in) {
+        if (!v.fn_in || ni > WS_INLINE)
+            return cudaErrorInvalidValue;
+        return launch_maybe_pdl(v.fn_in, grid, JT + 32, v.smem, s, pdl, a, *in);
+    }
+    return launch_maybe_pdl(v.fn, grid, JT + 32, v.smem, s, pdl, a, WsNone{});
+}
+
+bool ws_takes_inline(const ForceConfig &cfg)
+{
+    const int k = cfg.variant - (variant_count() - kNumWs);
+    return cfg.ws && k >= 0 && k < kNumWs && kWs[k].fn_in != nullptr;
 }
 
 }  // namespace g6
