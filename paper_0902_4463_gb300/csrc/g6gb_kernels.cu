@@ -284,6 +284,18 @@ __device__ __forceinline__ float2 ds_sep2(float2 h, float2 l, float2 nh, float2 
 // issue two lanes of FP32 work per instruction.  Subtractions are additions
 // of the pre-negated i values (exact).
 //
+// What bounds the loop: the FMA pipe and the register file behind it.  A
+// packed multiply-add with three distinct operands takes three cycles of
+// register reads where its arithmetic takes two (a microbenchmark reaches 80
+// of 128 lane operations per clock and SM, 105 with one operand shared by
+// neighbours, 120 for packed additions), and eleven of the 32 operations per
+// pair are such; a copy of this loop with real operands and nothing around
+// it reaches 0.74-0.76 of the FP32 peak at 60 operations per pair.  Measured
+// here: 0.77 at m = N = 2^20 (wide shape, eight waves), 0.71 at m = 2048, 0.65
+// at m = 251, where the CTAs of an SM end at different times.  More
+// i-particles per thread, other statement orders, loose warps and 512-thread
+// CTAs did not pass that bound.
+//
 // The j-groups take contiguous shares of a tile, so that the loads of two
 // j-pairs merge into 16-byte ones (strided shares: 3-7 % slower) and a
 // group's j-slots ascend; batches, whose entries are short, keep strided
@@ -1872,10 +1884,10 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
     // line would hold too few (i-tile, j-tile) units for the SMs: wide
     // tiles need many j-tiles to keep every CTA busy, so small j-sets
     // take narrower tiles at the same m.  (The 256-wide tile from 65536
-    // units on, measured with Plummer spheres: at N = 131072 the 128-wide
-    // split-j tile is 9 % faster for m = 8192 and 2 % for m = 32768, the
-    // wide one 4 % faster for m = 65536; at N = 32768, m = N the split-j
-    // tile is 16 % faster; at N = 2^20, m = 4096 the wide one by 1 %.)
+    // units on; force + reduction, us, wide and 128-wide split-j, each in
+    // its best number of waves: N = 131072: m = 8192: 1229 and 1183, m =
+    // 16384: 2276 and 2293, m = 40000: 5446 and 5509; N = 32768, m = 4096:
+    // 260 and 184; N = 2^20, m = 2048: 2281 either way.)
     struct Shape {
         int v, itile, max_ni;
         long long min_units;
