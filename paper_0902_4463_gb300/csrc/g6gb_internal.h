@@ -207,8 +207,9 @@ cudaError_t launch_reduce_batch(int v, int grid, const void *part, const int *ji
                                 g6x_out *d_out, const BatchTables &bt, int blocks,
                                 cudaStream_t s, bool fused = false);
 
-// The warp-specialised small-block variants (g6gb_small.cu) follow the
-// others in one numbering: variant_count() covers both tables.
+// The warp-specialised small-block variants (g6gb_small.cu) are WS_FIRST and
+// up in one numbering with the others: variant_count() covers both tables.
+constexpr int WS_FIRST = 28;
 int variant_count();
 VariantInfo variant_info(int v);
 int ws_variant_count();

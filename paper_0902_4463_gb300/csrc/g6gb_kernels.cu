@@ -1667,11 +1667,23 @@ const Variant kVariants[] = {
     {{16, 16, 2, 1, G6X_PREC_DS}, k_force_ds<16, 16, 2, true, 2, 2>, 256, ds_smem(256, 2)},
     {{32, 8, 2, 1, G6X_PREC_DS}, k_force_ds<32, 8, 2, true, 2, 2>, 256, ds_smem(256, 2)},
     {{64, 4, 2, 1, G6X_PREC_DS}, k_force_ds<64, 4, 2, true, 2, 2>, 256, ds_smem(256, 2)},
-    // FP64, narrow i-tiles
+    // FP64, narrow i-tiles (numbered after the small-block shapes)
     {{16, 8, 1, 0, G6X_PREC_FP64}, k_force_64<8, false>, 128, 0},
     {{8, 16, 1, 0, G6X_PREC_FP64}, k_force_64<16, false>, 128, 0},
 };
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
+
+// Variant numbers stand in saved tuning tables, so they stay: the shapes of
+// the small-block kernel follow the first WS_FIRST of this table, the rest of
+// this table follows them.  table_slot() is the index here of variant v, -1
+// if it is none of these.
+int table_slot(int v)
+{
+    const int nws = ws_variant_count();
+    if (v < 0 || v >= kNumVariants + nws || (v >= WS_FIRST && v < WS_FIRST + nws))
+        return -1;
+    return v < WS_FIRST ? v : v - nws;
+}
 
 // Batch force kernels: the same pair loop over the batch work geometry.
 const Variant kBatchVariants[] = {
@@ -1706,6 +1718,7 @@ void pin_carveout(F *fn)
     }
 }
 
+// v is an index into kVariants
 cudaError_t prepare_variant(int v)
 {
     if (!g_smem_set[v]) {
@@ -1732,25 +1745,25 @@ int variant_count() { return kNumVariants + ws_variant_count(); }
 
 VariantInfo variant_info(int v)
 {
-    return v < kNumVariants ? kVariants[v].info : ws_variant_info(v - kNumVariants);
+    const int k = table_slot(v);
+    return k >= 0 ? kVariants[k].info : ws_variant_info(v - WS_FIRST);
 }
 
 int variant_occupancy(int v)
 {
-    if (v >= kNumVariants)
-        return ws_variant_occupancy(v - kNumVariants);
-    if (v < 0)
-        return 0;
-    if (g_occ[v] == 0) {
-        if (prepare_variant(v) != cudaSuccess)
+    const int k = table_slot(v);
+    if (k < 0)
+        return ws_variant_occupancy(v - WS_FIRST);
+    if (g_occ[k] == 0) {
+        if (prepare_variant(k) != cudaSuccess)
             return 0;
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &n, kVariants[v].fn, kVariants[v].threads, kVariants[v].smem) != cudaSuccess)
+                &n, kVariants[k].fn, kVariants[k].threads, kVariants[k].smem) != cudaSuccess)
             return 0;
-        g_occ[v] = n;
+        g_occ[k] = n;
     }
-    return g_occ[v];
+    return g_occ[k];
 }
 
 // ------------------------------------------------------------- tuning ---
@@ -1848,11 +1861,11 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
             return 8;
         // the FP64 pipe pays for every lane, so the i-tile that pads the
         // block least (ties to the widest; large blocks pad little either way)
-        static constexpr int shapes64[] = {7, 28, 29};
+        const int nws = ws_variant_count();
         int best = 7;
         if (ni <= 256)
-            for (int v : shapes64) {
-                const int w = kVariants[v].info.ti, u = kVariants[best].info.ti;
+            for (int v : {WS_FIRST + nws, WS_FIRST + nws + 1}) {
+                const int w = variant_info(v).ti, u = variant_info(best).ti;
                 if ((ni + w - 1) / w * w < (ni + u - 1) / u * u)
                     best = v;
             }
@@ -1878,7 +1891,7 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
             }
         }
         if (best >= 0)
-            return kNumVariants + best;
+            return WS_FIRST + best;
     }
     // The widest i-tile the block size allows, narrowed while the work
     // line would hold too few (i-tile, j-tile) units for the SMs: wide
@@ -1990,7 +2003,7 @@ ForceConfig choose_config(int prec, int ni, int nj_pad, int list, int sm_count,
     c.jtiles = nj_pad / JT;
     c.n_itile = (ni + c.itile - 1) / c.itile;
     c.work = (long long)c.n_itile * c.jtiles;
-    c.smem = vi.ws ? ws_variant_smem(v - kNumVariants) : kVariants[v].smem;
+    c.smem = vi.ws ? ws_variant_smem(v - WS_FIRST) : kVariants[table_slot(v)].smem;
     c.list = vi.list;
     c.prec = vi.prec;
     c.ws = vi.ws;
@@ -2092,9 +2105,10 @@ cudaError_t launch_update_predict(int kind, JStore js, Pred p, int nj, int nj_pa
 // Arguments of the fused prediction (variants with fpred set).
 static bool set_fused_pred(ForceArgs &a, const ForceConfig &cfg, const FusedPred *fp)
 {
-    if (cfg.ws || cfg.variant < 0 || cfg.variant >= kNumVariants)
+    const int k = table_slot(cfg.variant);
+    if (cfg.ws || k < 0)
         return false;
-    if (!kVariants[cfg.variant].info.fpred)
+    if (!kVariants[k].info.fpred)
         return true;
     if (!fp)
         return false;
@@ -2115,9 +2129,10 @@ cudaError_t launch_force(const ForceConfig &cfg, const Pred &p,
 {
     if (cfg.work <= 0)
         return cudaSuccess;
-    if (cfg.ws || cfg.variant < 0 || cfg.variant >= kNumVariants)
+    const int k = table_slot(cfg.variant);
+    if (cfg.ws || k < 0)
         return cudaErrorInvalidValue;           // small-block kernel: launch_force_ws
-    cudaError_t e = prepare_variant(cfg.variant);
+    cudaError_t e = prepare_variant(k);
     if (e != cudaSuccess)
         return e;
     ForceArgs a{};
@@ -2146,7 +2161,7 @@ cudaError_t launch_force(const ForceConfig &cfg, const Pred &p,
     a.wait_ns = g_wait_ns;
     if (!set_fused_pred(a, cfg, fp))
         return cudaErrorInvalidValue;
-    const Variant &v = kVariants[cfg.variant];
+    const Variant &v = kVariants[k];
     return launch_maybe_pdl(v.fn, cfg.grid, v.threads, v.smem, s, pdl, a);
 }
 
@@ -2158,13 +2173,14 @@ cudaError_t launch_force_fused(const ForceConfig &cfg, const Pred &p,
 {
     if (cfg.work <= 0)
         return cudaSuccess;
-    if (cfg.prec != G6X_PREC_DS || cfg.ws || cfg.variant < 0 || cfg.variant >= kNumVariants)
+    const int k = table_slot(cfg.variant);
+    if (cfg.prec != G6X_PREC_DS || cfg.ws || k < 0)
         return cudaErrorInvalidValue;
     if (cfg.list
         && (!lists || !lists->nbmax || lists->nbseg < 1 || lists->nbseg > lists->maxnb
             || !lists->nbl_part || !lists->nbc_part || !lists->nbl_out || !lists->nblen_out))
         return cudaErrorInvalidValue;
-    cudaError_t e = prepare_variant(cfg.variant);
+    cudaError_t e = prepare_variant(k);
     if (e != cudaSuccess)
         return e;
     ForceArgs a{};
@@ -2197,7 +2213,7 @@ cudaError_t launch_force_fused(const ForceConfig &cfg, const Pred &p,
     }
     if (!set_fused_pred(a, cfg, fp))
         return cudaErrorInvalidValue;
-    const Variant &v = kVariants[cfg.variant];
+    const Variant &v = kVariants[k];
     return launch_maybe_pdl(v.fn, cfg.grid, v.threads, v.smem, s, pdl, a);
 }
 

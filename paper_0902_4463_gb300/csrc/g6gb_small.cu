@@ -933,7 +933,7 @@ cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int 
                             int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl,
                             const WsInline *in)
 {
-    const int k = cfg.variant - (variant_count() - kNumWs);
+    const int k = cfg.variant - WS_FIRST;
     const int grid = cfg.grid, jtiles = cfg.jtiles;
     if (!cfg.ws || k < 0 || k >= kNumWs || grid < 1 || grid > jtiles || ni < 1
         || ni > kWs[k].info.ti * kWs[k].info.nper)
@@ -969,7 +969,7 @@ cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int 
 
 bool ws_takes_inline(const ForceConfig &cfg)
 {
-    const int k = cfg.variant - (variant_count() - kNumWs);
+    const int k = cfg.variant - WS_FIRST;
     return cfg.ws && k >= 0 && k < kNumWs && kWs[k].fn_in != nullptr;
 }
 
