@@ -1935,19 +1935,20 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
     // CTAs, so equal shares of the work line finish at different times, and
     // with one wave the SMs run their last stretch with few warps.  Later
     // waves fill those slots.  More CTAs also mean more partial records and
-    // i-tile loads, so the count follows the length of the work line.
+    // i-tile loads, so the count rises with the length of the work line and
+    // never falls.
     const long long units =
         (long long)((ni + shapes[k].itile - 1) / shapes[k].itile) * jtl;
-    if (shapes[k].v == 23) {
-        *gmul = units < (1LL << 18) ? 1 : units < (1LL << 21) ? 2 : units < (1LL << 23) ? 4 : 8;
-    } else if (shapes[k].v == 9) {
-        // measured (force + reduction, ms): 40000 x 131072 (80384 units) 5.53,
-        // 5.46 and 5.45 in 1, 2 and 4 waves; 16384 x 2^20 16.93 in 2, 16.96 in
-        // 8; 65536 x 2^20 67.4, 66.7 and 66.5 in 2, 4 and 8; 4096 x 2^20
-        // (65536 units) 4.39 in 1, 4.38 in 4; 2^18 x 2^20 265.8 in 4, 264.9
-        // in 8; 2^20 x 2^20 1058 in 8
-        *gmul = units <= (1LL << 16) ? 1 : units < (1LL << 19) ? 2
-                : units < (1LL << 21) || units >= (1LL << 23) ? 8 : 4;
+    if (shapes[k].itile == 256) {
+        // measured (whole step, N = 2^20, ms, in 1, 2, 4 and 8 waves):
+        // m = 4096 (2^16 units) 4.388, 4.349, 4.378, 4.563; 8192 8.67, 8.53,
+        // 8.55, 8.65; 16384 17.24, 16.92, 16.82, 16.95; 65536 (2^20 units)
+        // 68.5, 67.3, 66.6, 66.4; 131072 136.8, 134.2, 133.1, 132.6; 262144
+        // (2^22 units) 273.6, 268.2, 265.5, 264.7; N = m = 131072 17.52,
+        // 17.16, 17.16, 17.19.  The fastest count rises 2, 4, 8; below 2^23
+        // units the rule takes fewer, which costs 0.3-1.6 % and saves partial
+        // records (m = 65536: 27 MB of them in 2 waves, 94 MB in 8)
+        *gmul = units < (1LL << 17) ? 1 : units < (1LL << 21) ? 2 : units < (1LL << 23) ? 4 : 8;
     } else if (shapes[k].v == 16) {
         // measured (us): 512 x 2^20 (16384 units) 611 in 1 wave, 603 in 2;
         // 6000 x 131072 896 and 885; 2048 x 2^20 (65536 units) 2345, 2291 and
