@@ -787,8 +787,8 @@ int run_force(Ctx &c, const ForceConfig &cfg, int nj, int ni, const g6x_irec *d_
         if (rc)
             return rc;
         PhaseTimer pt(c, PH_FORCE);
-        e = g6::launch_force_ws(cfg, d_irec, ni, eps2, nj, c.d_part, c.d_tcnt, d_out, c.js.idx,
-                                c.d_err, fpa, c.stream, pdl, in);
+        e = g6::launch_force_ws(cfg, d_irec, ni, eps2, nj, c.d_part, c.d_tcnt, d_out, c.d_err,
+                                fpa, c.stream, pdl, in);
         c.launches += 1;
     } else if (cfg.prec == G6X_PREC_DS && seg_per_tile <= g6::FUSED_MAX_SEGS) {
         // one launch: the last CTA of each i-tile reduces it (K3 fused into
@@ -1657,7 +1657,7 @@ extern "C" int g6x_autotune(int cid, int nj, int m_max, const char *path)
                                                c->sm_count, c->stream);
                     if (e == cudaSuccess && vi.ws) {
                         e = g6::launch_force_ws(cfg, d_i, m, 1e-6, nj, c->d_part, c->d_tcnt, d_o,
-                                                c->js.idx, c->d_err, fpa, c->stream, false);
+                                                c->d_err, fpa, c->stream, false);
                     } else {
                         if (e == cudaSuccess)
                             e = g6::launch_force(cfg, c->pred, d_i, m, 1e-6, c->d_part, nullptr,

@@ -291,8 +291,8 @@ cudaError_t launch_force_fused(const ForceConfig &cfg, const Pred &p,
 // into out; part holds partial_slots(cfg) records, cnt counter_slots(cfg)
 // counters, zero before the launch and left zero by a launch that completes.
 cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int ni, double eps2,
-                            int nj, void *part, unsigned *cnt, g6x_out *out, const int *jidx,
-                            int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl,
+                            int nj, void *part, unsigned *cnt, g6x_out *out, int *d_err,
+                            const FusedPred &fp, cudaStream_t s, bool pdl,
                             const WsInline *in = nullptr);
 // Whether launch_force_ws takes this launch's records from `in` (i-tiles of
 // up to WS_INLINE; then d_irec, fp.rec and fp.toff are not read).

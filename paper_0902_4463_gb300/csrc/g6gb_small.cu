@@ -929,9 +929,8 @@ size_t ws_partial_slots(int grid, int itile)
 }
 
 cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int ni, double eps2,
-                            int nj, void *part, unsigned *cnt, g6x_out *out, const int *jidx,
-                            int *d_err, const FusedPred &fp, cudaStream_t s, bool pdl,
-                            const WsInline *in)
+                            int nj, void *part, unsigned *cnt, g6x_out *out, int *d_err,
+                            const FusedPred &fp, cudaStream_t s, bool pdl, const WsInline *in)
 {
     const int k = cfg.variant - WS_FIRST;
     const int grid = cfg.grid, jtiles = cfg.jtiles;
@@ -948,7 +947,6 @@ cudaError_t launch_force_ws(const ForceConfig &cfg, const g6x_irec *d_irec, int 
     a.ni = ni;
     a.eps2 = eps2;
     a.out = out;
-    a.jidx = jidx;
     a.tcnt = cnt;
     a.fused = 1;
     a.wait_ns = wait_limit_ns();
