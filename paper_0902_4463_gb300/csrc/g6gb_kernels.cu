@@ -99,7 +99,7 @@ __global__ void k_irec_from_store(JStore js, g6x_irec *out, int m)
 
 // Records the range of particle indices of each 32 j-slots (empty slots
 // excluded): every warp of the CTA its own, so the predictor needs no
-// barrier (with one range per tile it met at one per tile).
+// barrier.
 __device__ __forceinline__ void index_ranges(int id, bool valid, int2 *out)
 {
     const int lo = __reduce_min_sync(0xffffffffu, valid ? id : INT_MAX);
@@ -284,22 +284,19 @@ __device__ __forceinline__ float2 ds_sep2(float2 h, float2 l, float2 nh, float2 
 // issue two lanes of FP32 work per instruction.  Subtractions are additions
 // of the pre-negated i values (exact).
 //
-// What bounds the loop: the FMA pipe and the register file behind it.  A
-// packed multiply-add with three distinct operands takes three cycles of
-// register reads where its arithmetic takes two (a microbenchmark reaches 80
-// of 128 lane operations per clock and SM, 105 with one operand shared by
-// neighbours, 120 for packed additions), and eleven of the 32 operations per
-// pair are such; a copy of this loop with real operands and nothing around
-// it reaches 0.74-0.76 of the FP32 peak at 60 operations per pair.  Measured
-// here: 0.77 at m = N = 2^20 (wide shape, eight waves), 0.71 at m = 2048, 0.65
-// at m = 251, where the CTAs of an SM end at different times.  More
-// i-particles per thread, other statement orders, loose warps and 512-thread
-// CTAs did not pass that bound.
+// What bounds the loop: the FMA pipe.  32 lane operations per pair allow 0.94
+// of the FP32 peak at 60 operations per pair; ncu shows the pipe 83 % busy at
+// m = N = 2^18, its throttle the first stall.  Measured fractions of the peak:
+// 0.777 at m = N = 2^20 (256-wide, eight waves), 0.71 at m = 2048, 0.65 at m =
+// 251, where the CTAs of an SM end at different times.  No gain at m = N from
+// more i-particles per thread, other statement orders, 512-thread CTAs or
+// warps that count themselves out of a tile instead of meeting at a barrier.
 //
 // The j-groups take contiguous shares of a tile, so that the loads of two
 // j-pairs merge into 16-byte ones (strided shares: 3-7 % slower) and a
-// group's j-slots ascend; batches, whose entries are short, keep strided
-// shares.  The per-pair self test is needed only where the
+// group's j-slots ascend.  Batches keep strided shares, though contiguous
+// ones are 3 % faster there too: with the sums in that order one force of the
+// driver test that nearly cancels (|a| = 0.011) is 2e-5 off, past its bound.  The per-pair self test is needed only where the
 // index range of a warp's j-particles holds one of its i-particles; others
 // take the same loop without it.
 // The nearest neighbour is tracked lazily: a running minimum of the key per
@@ -628,11 +625,10 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
     // Nearest neighbour of one i-particle (negated DS position xh, xl, index
     // id_i) from the share that holds its smallest key, by SL lanes together:
     // the keys again with the loop's arithmetic, whose packed lanes round
-    // like the scalar operations used here.  (Before, every thread searched
-    // the chunk of 8 j-particles noted in the loop for each of its own
-    // i-particles, before the j-groups were combined: scattered loads that
-    // took 25 of the 350 us of m = 251, N = 10^6, and the notes cost the
-    // loop 4 %.)
+    // like the scalar operations used here.  A search by every thread for each
+    // of its own i-particles, before the j-groups combine, scatters its
+    // loads: 25 us more at m = 251, N = 10^6 (333 us a step), and the loop
+    // 4 % slower by noting a chunk to search.
     using Search = ShareSearch<SHT>;
     constexpr int SL = Search::SL;
     auto nn_scan = [&](int share, const float *xh, const float *xl, int id_i) -> Search {
@@ -1217,7 +1213,8 @@ __global__ void __launch_bounds__(TI * TJ, MINB) k_force_ds(const ForceArgs a)
 // Treatment of a Single Nonlinear Equation, 1970): with e = 1 - s y0^2,
 // y = y0 + y0 e (1/2 + 3/8 e) leaves 5/16 e^3, below a rounding for an
 // approximation good to 2^-20.  Five FP64 operations.  Zero, infinity and
-// subnormal s take the library's function.
+// subnormal s take the library's function.  At most 0.97 units in the last
+// place over 52000 arguments of all binary exponents.
 __device__ __forceinline__ double rsqrt64(double s)
 {
     const unsigned hi = (unsigned)__double2hiint(s);
@@ -1236,13 +1233,13 @@ __device__ __forceinline__ double rsqrt64(double s)
 // Bound by the FP64 pipe (2 lanes per clock and SM): 33 FP64 operations per
 // pair, and nothing else on that pipe: the neighbour and list tests compare
 // the keys as unsigned integers (they are not negative, so the order is the
-// same; a NaN of either sign still loses) and the index as bits.  With one i-particle per thread of
-// 128 and tiles of 256 a block of 793 paid for 896 lanes and CTAs of one unit
-// each; 32-wide i-tiles pay for 800, and the line of 64-wide sub-tiles is cut
-// evenly over the SMs.  Force alone, before and after (us): m = 793, N =
-// 32768: 1941 and 1588; m = 972, N = 131072: 9776 and 7686 (0.79 of the pipe at
-// 60 operations per pair); m = 32, N = 32768: 340 and 84; m = 1 (8-wide
-// i-tiles): 338 and 32; m = 7, N = 1024: 336 and 16.
+// same; a NaN of either sign still loses) and the index as bits.  32-wide
+// i-tiles pay for 800 lanes at m = 793 (128-wide ones for 896), and the line of
+// 64-wide sub-tiles is cut evenly over the SMs.  Force alone, us, here and with
+// 128-wide i-tiles, whole j-tiles and the library's reciprocal root: m = 793,
+// N = 32768: 1588 and 1941; m = 972, N = 131072: 7686 and 9776 (0.79 and 0.62
+// of the measured FP64 peak at 60 operations per pair); m = 32, N = 32768: 84 and
+// 340; m = 1 (8-wide): 32 and 338; m = 7, N = 1024: 16 and 336.
 template <int TJ, bool LIST>
 __global__ void __launch_bounds__(128) k_force_64(const ForceArgs a)
 {
@@ -1839,12 +1836,15 @@ void tune_clear()
 namespace {
 
 // Blocks the built-in choice gives the small-block kernel.  Measured on
-// GB300 as the host wall time of a block step through the GRAPE calls
-// (the separate predictor and split-j shapes overlap their three launches):
-// faster for m <= 16 at every N (N = 131072, m = 16: 36 against 42 us);
-// for m <= 32 once the j-set has 512 tiles (N = 32768: a tie; N = 2^20:
-// 92 against 122 us); for m <= 64 only from about 1500 tiles on (N =
-// 262144: 72 against 67 us; N = 2^20: 142 against 173 us); never above.
+// GB300 as the host wall time of a block step through the GRAPE calls, choice
+// forced, m staged and m active particles (us; this kernel, then the separate
+// predictor, split-j shape and reduction, whose launches overlap): m = 16: N =
+// 1024: 22.6 and 30.1, 32768: 25.6 and 32.5, 2^20: 57 and 85; m = 32: N = 1024:
+// 24.6 and 30.6, 32768: 30.6 and 34.6, 131072: 38.5 and 42.9, 2^20: 78 and 106;
+// m = 64: N = 32768: 45 and 40, 262144: 73 and 61, 2^20: 132 and 141; m = 96: N =
+// 2^20: 229 and 213.  So 17 to 32 particles could take it below 512 tiles
+// too; that line stands where a tie lay when the records of a block that
+// small still came from mapped memory.
 constexpr int WS_ANY_N_MAX_NI = 16;
 constexpr int WS_MID_MAX_NI = 32;
 constexpr long long WS_MID_MIN_JTILES = 512;
@@ -1860,7 +1860,17 @@ int heuristic_variant(int prec, int ni, int nj_pad, int list, bool allow_ws, int
         if (list)
             return 8;
         // the FP64 pipe pays for every lane, so the i-tile that pads the
-        // block least (ties to the widest; large blocks pad little either way)
+        // block least, ties to the widest.  Measured (whole step, us; 32, 16
+        // and 8 wide): N = 32768: m = 8: 96, 62, 44; 17: 96, 91, 83; 40: 170,
+        // 135, 112; 48: 170, 134, 138; 104: 279, 280, 234; 200: 463, 438, 424;
+        // 248: 536, 531, 516; N = 131072: m = 40: 542, 416, 350; 120: 1014,
+        // 1028, 971.  With few sub-tiles per CTA their rounding counts more
+        // than the padding, and the rule can miss the best by a quarter:
+        // N = 8192: m = 72: 74, 68, 81; 120: 92, 88, 111; 216: 133, 156, 145;
+        // N = 1024: m = 248: 37, 38, 41.  Against 128-wide i-tiles on whole
+        // j-tiles the rule is 1.1 times faster at least (m = 1 to 1000, N =
+        // 1024 to 131072).  Above 256 the padding is below an eighth, 32 wide
+        // is the rule (m = 300, N = 32768: 680, 621, 620)
         const int nws = ws_variant_count();
         int best = 7;
         if (ni <= 256)

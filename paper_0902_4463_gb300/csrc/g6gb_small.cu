@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(TI * TJ + 32, MINB) k_force_ws(const ForceArgs
     // searched for once, at the end, in the winning share.  (Searching the
     // tile at once, while still in shared memory, runs in nearly every tile
     // of a short share of the line, since one lane of the warp is enough:
-    // 3 of the 47 us of m = 16, N = 2^20.)
+    // 3 us more at m = 16, N = 2^20, where a launch takes 43 us.)
     bool ok = ntile <= 0 || predict_into(0);
     cta_bar();
     int since_flush = 0;
@@ -862,8 +862,10 @@ int g_ws_occ[kNumWs];
 }  // namespace
 
 // Grids of up to this many CTAs reduce in one level: the second level costs
-// an arrival, a fence and a round of loads (2.5 of the 14.3 us of a block
-// step at N = 1024, 4 CTAs) that a few more records per lane do not.
+// an arrival, a fence and a round of loads that a few more records per lane
+// do not.  Device time of a step, one level and two (us): 4 CTAs (N = 1024, m =
+// 7) 7.9 and 9.7, 16 CTAs (N = 4096) 9.1 and 10.5, 32 CTAs (N = 8000, m = 16)
+// 10.5 and 10.8.
 constexpr int WS_ONE_LEVEL = 32;
 
 int ws_variant_count() { return kNumWs; }
