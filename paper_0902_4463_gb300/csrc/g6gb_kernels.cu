@@ -285,10 +285,10 @@ __device__ __forceinline__ float2 ds_sep2(float2 h, float2 l, float2 nh, float2 
 // of the pre-negated i values (exact).
 //
 // What bounds the loop: the FMA pipe.  32 lane operations per pair allow 0.94
-// of the FP32 peak at 60 operations per pair; ncu shows the pipe 83 % busy at
-// m = N = 2^18, its throttle the first stall.  Measured fractions of the peak:
-// 0.777 at m = N = 2^20 (256-wide, eight waves), 0.71 at m = 2048, 0.65 at m =
-// 251, where the CTAs of an SM end at different times.  No gain at m = N from
+// of the FP32 peak at 60 operations per pair; ncu shows the pipe 82 % busy at
+// m = N = 2^18, its throttle the first stall.  Measured fractions of the peak at
+// N = 2^20: 0.777 at m = N (256-wide, eight waves), 0.71 at m = 2048, 0.65 at m =
+// 256, where the CTAs of an SM end at different times.  No gain at m = N from
 // more i-particles per thread, other statement orders, 512-thread CTAs or
 // warps that count themselves out of a tile instead of meeting at a barrier.
 //
